@@ -46,7 +46,7 @@ void free_ctx(Context* c) {
                   c->items,   c->item_part, c->extra,   c->work_ctr,   c->vt,            c->it,
                   c->bvh_parent, c->bvh_valid, c->bvh_keys, c->bvh_flags, c->bvh_bounds, c->bvh_bad,
                   c->bvh_mode, c->extra64, c->ct_partials, c->dedge, c->ovf_list, c->acc_fx, c->act_off,
-                  c->trace_list, c->st_done, c->cand_st, c->bin_cnt, c->bvh_stale, c->bvh_need};
+                  c->trace_list, c->st_done, c->cand_st, c->bin_cnt, c->bvh_stale, c->bvh_need, c->pool_pm, c->face_rec};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete[] c->hvt;
@@ -111,7 +111,7 @@ int create_ctx(const hr_limits* lim, int n, size_t views, size_t subtiles, size_
   const size_t nviews = views;
   bool ok = dev_alloc(&c->nodes, ni * F, a) && dev_alloc(&c->tris, ni * 3 * F, a) &&
             dev_alloc(&c->normals, ni * 3 * V, a) && dev_alloc(&c->normal_len, ni * V, a) &&
-            dev_alloc(&c->partials, partial_blocks * 6 * V, a) && dev_alloc(&c->dN, ni * 3 * V, a) &&
+            dev_alloc(&c->partials, partial_blocks * 8 * V, a) && dev_alloc(&c->dN, ni * 3 * V, a) &&
             dev_alloc(&c->dedge, ni * 3 * V, a) && dev_alloc(&c->acc_fx, ni * 6 * V, a) &&
             dev_alloc(&c->sil, nviews * lim->max_E, a) &&
             dev_alloc(&c->sil_count, nviews, a) &&
@@ -119,9 +119,10 @@ int create_ctx(const hr_limits* lim, int n, size_t views, size_t subtiles, size_
             dev_alloc(&c->counters, ni * 4, a) && dev_alloc(&c->skin_partials, ni * hr::kSkinBlocks * hr::kSkinAcc, a) &&
             dev_alloc(&c->status, 1, a) && dev_alloc(&c->stats, 3 * hr::kStatsPer, a) &&
             dev_alloc(&c->pool_bb, c->pool_cap, a) && dev_alloc(&c->pool_z, c->pool_cap, a) &&
-            dev_alloc(&c->pool_rec, c->pool_cap, a) && dev_alloc(&c->st_info, subtiles, a) &&
+            dev_alloc(&c->pool_rec, c->pool_cap, a) &&
+            dev_alloc(&c->pool_pm, c->pool_cap, a) && dev_alloc(&c->face_rec, ni * F * hr::kFaceRec, a) && dev_alloc(&c->st_info, subtiles, a) &&
             dev_alloc(&c->items, c->item_cap, a) && dev_alloc(&c->item_part, (size_t)c->item_cap * 32, a) &&
-            dev_alloc(&c->extra, ni * 6 * V, a) && dev_alloc(&c->work_ctr, hr::ctr_words(ni), a) &&
+            dev_alloc(&c->extra, ni * 8 * V, a) && dev_alloc(&c->work_ctr, hr::ctr_words(ni), a) &&
             dev_alloc(&c->ovf_list, subtiles, a) && dev_alloc(&c->trace_list, c->item_cap, a) &&
             dev_alloc(&c->st_done, subtiles, a) && dev_alloc(&c->cand_st, subtiles, a) &&
             dev_alloc(&c->bin_cnt, subtiles, a) &&

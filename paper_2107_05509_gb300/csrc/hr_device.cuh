@@ -121,12 +121,14 @@ struct Context {
   float4* pool_bb;       // [pool_cap]
   float* pool_z;         // [pool_cap]
   int* pool_rec;         // [pool_cap]
+  unsigned* pool_pm;     // [pool_cap]
+  float4* face_rec;      // [n_inst][max_F][kFaceRec] shading records (k_bin, k_items_bwd)
   int pool_cap;
   int2* st_info;         // [sub-tiles]
   int4* items;           // [item_cap], one region per instance
   float4* item_part;     // [item_cap][32]
   int item_cap;
-  float* extra;          // [n_inst][max_V][6]
+  float* extra;          // [n_inst][max_V][8]
   double* extra64;       // [n_inst][max_V][6] backward sums when max_V > 8192
   unsigned* work_ctr;    // [3 + 2 n_inst]
   int* ovf_list;         // [sub-tiles] sub-tiles whose items overflowed their region
@@ -135,7 +137,7 @@ struct Context {
   int4* cand_st;         // [sub-tiles] forward lists to sort: (sub-tile, pool offset, K, 0)
   unsigned* bin_cnt;     // [sub-tiles] records binned per sub-tile (zeroed by every forward)
   // backward scratch
-  float* partials;       // [render_blocks][max_V][6] (single-instance contexts)
+  float* partials;       // [num_sms][max_V][8] (single-instance contexts)
   float* dN;             // [n_inst][max_V][3]
   float* dedge;          // [n_inst][max_V][3] the edge-sampling term's vertex sums
   unsigned long long* acc_fx;   // [n_inst][max_V][6] fixed-point backward sums (HR_DETERMINISTIC)
@@ -182,6 +184,8 @@ constexpr int kLossBlocks = 304;         // loss blocks of a single-instance con
 constexpr int kLossBlocksBatch = 128;    // per instance in a batch
 // per-instance loss scratch: block counts (u64), block sums, 1 / (3 sum M), padding
 __host__ __device__ constexpr int kLossStride(int blocks) { return 4 * blocks + 8; }
+// float4 words of a face's shading record (write_face_record in hr_render.cu)
+constexpr int kFaceRec = 9;
 constexpr int kStatsPer = 6;   // samples, rays, BVH nodes, triangle tests, hits, candidate box tests
 constexpr int kSkinBlocks = 64;
 constexpr int kSkinAcc = 16 * 12 + 10 + 3;   // dA_j (J=16 x 3x4), dbeta, dtau

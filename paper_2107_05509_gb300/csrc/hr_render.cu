@@ -20,13 +20,14 @@
 // when the forward's cannot be reused.
 //
 // Shading:
-//   k_shade_fwd    warps take work items; each lane (pixel) makes its samples
-//                  (Philox jitter) and walks the candidates that can hold a sample of
-//                  its pixel (a bit transpose of the warp's box-against-pixel tests),
-//                  in depth order, with the same float32 Moller-Trumbore test and
-//                  closest-hit rule as a per-ray traversal, stopping at the first
-//                  candidate nearer than none of its hits; shades, and writes per-item
-//                  sums.  The warp finishing a sub-tile's last item sums the items in
+//   k_shade_fwd    warps take work items; the warp stages the item's candidates in
+//                  shared memory (what their intersection needs, the camera's part
+//                  already worked out), each lane (pixel) makes its samples (Philox
+//                  jitter) and walks the candidates that can cover its pixel (a bit
+//                  transpose of the lists' pixel masks), in depth order, with the same
+//                  float32 Moller-Trumbore test and closest-hit rule as a per-ray
+//                  traversal, stopping at the first candidate nearer than none of its
+//                  hits; shades, and writes per-item sums.  The warp finishing a sub-tile's last item sums the items in
 //                  item order (deterministic) and writes the pixels.
 //   k_shade_bwd    the same samples re-traced (no hit records are kept between
 //                  the passes); every hit is differentiated at the fixed ray and the
@@ -60,6 +61,7 @@ namespace {
 
 constexpr int kRenderThreads = 128;   // 4 warps per block
 constexpr int kWarps = kRenderThreads / 32;
+constexpr int kFwdMinBlocks = 7;      // launch bound of the forward shader (72 registers)
 constexpr int kBwdMinBlocks = 4;      // launch bound of the backward shader (128 registers)
 constexpr int kBlocksPerSm = 8;       // largest persistent grid; backward partials are sized for it
 constexpr int kSubW = 8, kSubH = 4;   // sub-tile; lane = pixel
@@ -198,6 +200,7 @@ struct Work {
   float4* bb;      // [pool] screen box (x0, y0, x1, y1) of the candidate
   float* z;        // [pool] nearest camera depth (sorted within a sub-tile)
   int* rec;        // [pool] triangle record
+  unsigned* pm;    // [pool] pixels of the sub-tile (bit = lane) that the triangle can cover
   int pool_cap;
   int2* st;        // [sub-tiles] (pool offset, K): K = 0 no ray can hit, K < 0 per-ray
                    // traversal (-1: too many candidates; -(n + 1): n found no pool room)
@@ -206,7 +209,7 @@ struct Work {
   float4* part;    // [items][32] forward per-item sums (r, g, b, misses)
   double* extra64; // [n_inst][6V] backward sums of meshes beyond shared memory (float64
                    // atomics: long runs of cancelling contributions)
-  float* extra;    // [n_inst][6V] backward sums: shading blocks of a batch, and work
+  float* extra;    // [n_inst][8V] backward sums: shading blocks of a batch, and work
                    // done outside the shading blocks
   unsigned* ctr;   // [ctr_words(n_inst)] sub-tile counter, pool fill, per instance
                    // front items and taken items, the overflow count, per instance back
@@ -231,6 +234,7 @@ struct RenderArgs {
   const int* faces;
   const float* normals;    // instance i at + 3 i V
   const float* albedo;
+  float4* frec;            // shading records by face id; instance i at + kFaceRec i node_stride
   const Cam* cams;         // [views]
   const float* bg;
   int N, H, W, spp, V;     // uniform layout (single instance)
@@ -239,6 +243,7 @@ struct RenderArgs {
   const int* active;       // batch: instances with 0 are skipped (retired), or null
   const int* act_off;      // with `active`: [2][n_inst + 1] active sub-tile / view prefix sums
   int n_inst, nviews, total_st;
+  int num_sms;
   int node_stride;
   int cand_per_chunk, max_chunks;   // work-item split (tuning)
   const float* uv;        // [V][2] texture coordinates (shared by all instances)
@@ -260,13 +265,19 @@ struct RenderArgs {
 // four texels (clamped to the edge) and their weights
 struct TexSample {
   int i0, i1, j0, j1;
+  int cell;   // the unclamped corner (x + 1 in the low half, y + 1 above): -1 .. size each
   float fx, fy;
 };
-__device__ __forceinline__ TexSample tex_coords(const RenderArgs& a, int3 f, float u, float v) {
+__device__ __forceinline__ void tex_corners(const RenderArgs& a, TexSample& ts) {
+  const int xi = (ts.cell & 0xffff) - 1, yi = (ts.cell >> 16) - 1;
+  ts.i0 = min(max(xi, 0), a.tex_w - 1);
+  ts.i1 = min(max(xi + 1, 0), a.tex_w - 1);
+  ts.j0 = min(max(yi, 0), a.tex_h - 1);
+  ts.j1 = min(max(yi + 1, 0), a.tex_h - 1);
+}
+__device__ __forceinline__ TexSample tex_coords(const RenderArgs& a, float4 t01, float4 t2, float u, float v) {
   const float w = __fsub_rn(__fsub_rn(1.0f, u), v);
-  const float2 t0 = __ldg(reinterpret_cast<const float2*>(a.uv) + f.x);
-  const float2 t1 = __ldg(reinterpret_cast<const float2*>(a.uv) + f.y);
-  const float2 t2 = __ldg(reinterpret_cast<const float2*>(a.uv) + f.z);
+  const float2 t0 = make_float2(t01.x, t01.y), t1 = make_float2(t01.z, t01.w);
   const float ux = __fmaf_rn(v, t2.x, __fmaf_rn(u, t1.x, __fmul_rn(w, t0.x)));
   const float uy = __fmaf_rn(v, t2.y, __fmaf_rn(u, t1.y, __fmul_rn(w, t0.y)));
   const float x = __fmaf_rn(ux, (float)a.tex_w, -0.5f), y = __fmaf_rn(uy, (float)a.tex_h, -0.5f);
@@ -275,10 +286,8 @@ __device__ __forceinline__ TexSample tex_coords(const RenderArgs& a, int3 f, flo
   ts.fx = __fsub_rn(x, xf);
   ts.fy = __fsub_rn(y, yf);
   const int xi = (int)fminf(fmaxf(xf, -1.0f), (float)a.tex_w), yi = (int)fminf(fmaxf(yf, -1.0f), (float)a.tex_h);
-  ts.i0 = min(max(xi, 0), a.tex_w - 1);
-  ts.i1 = min(max(xi + 1, 0), a.tex_w - 1);
-  ts.j0 = min(max(yi, 0), a.tex_h - 1);
-  ts.j1 = min(max(yi + 1, 0), a.tex_h - 1);
+  ts.cell = (xi + 1) | ((yi + 1) << 16);
+  tex_corners(a, ts);
   return ts;
 }
 
@@ -295,9 +304,56 @@ __device__ __forceinline__ float3 tex_albedo(const RenderArgs& a, const TexSampl
                      gy * (gx * t00.z + ts.fx * t10.z) + ts.fy * (gx * t01.z + ts.fx * t11.z));
 }
 
+// Shading record of a face, kFaceRec float4 words:
+//   0-2  (n_k, vertex index k)   unit normals of the corners
+//   3-5  (albedo_k, e1 component k)
+//   6    (e2, v_0.x)
+//   7    (uv_0, uv_1)            (texture coordinates: with a texture)
+//   8    (uv_2, v_0.y, v_0.z)
+// A hit reads its face in a few 16-byte loads that depend on nothing but the face id,
+// instead of the indices and then 18 to 27 scalar loads behind them.  Rewritten by
+// every render call (from the current normals, albedo and vertices); an index outside
+// the model is taken as vertex 0 (the build has reported it).
+__device__ __forceinline__ void write_face_record(const RenderArgs& a, int f) {
+  int i[3];
+  float3 n[3], c[3], v[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    i[k] = __ldg(&a.faces[3 * f + k]);
+    if (i[k] < 0 || i[k] >= a.V) i[k] = 0;
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    n[k] = ld3(a.normals + 3 * i[k]);
+    c[k] = ld3(a.albedo + 3 * i[k]);
+    v[k] = ld3(a.verts + 3 * i[k]);
+  }
+  const float3 e1 = dsub(v[1], v[0]), e2 = dsub(v[2], v[0]);
+  float4* r = a.frec + (size_t)kFaceRec * f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) r[k] = make_float4(n[k].x, n[k].y, n[k].z, __int_as_float(i[k]));
+  r[3] = make_float4(c[0].x, c[0].y, c[0].z, e1.x);
+  r[4] = make_float4(c[1].x, c[1].y, c[1].z, e1.y);
+  r[5] = make_float4(c[2].x, c[2].y, c[2].z, e1.z);
+  r[6] = make_float4(e2.x, e2.y, e2.z, v[0].x);
+  float2 t2 = make_float2(0.0f, 0.0f);
+  if (a.tex) {
+    const float2* uv = reinterpret_cast<const float2*>(a.uv);
+    const float2 t0 = __ldg(uv + i[0]), t1 = __ldg(uv + i[1]);
+    t2 = __ldg(uv + i[2]);
+    r[7] = make_float4(t0.x, t0.y, t1.x, t1.y);
+  }
+  r[8] = make_float4(t2.x, t2.y, v[0].y, v[0].z);
+}
+
+// the records of every active instance, by all threads of the grid
+__device__ __forceinline__ void write_face_records(const RenderArgs& a);
+
+__device__ __forceinline__ float3 xyz(float4 q) { return make_float3(q.x, q.y, q.z); }
+
 __device__ __forceinline__ float3 shade(const RenderArgs& a, const Hit& h) {
-  int i0 = __ldg(&a.faces[3 * h.tri]), i1 = __ldg(&a.faces[3 * h.tri + 1]), i2 = __ldg(&a.faces[3 * h.tri + 2]);
-  float3 n0 = ld3(a.normals + 3 * i0), n1 = ld3(a.normals + 3 * i1), n2 = ld3(a.normals + 3 * i2);
+  const float4* r = a.frec + (size_t)kFaceRec * h.tri;
+  const float3 n0 = xyz(__ldg(r)), n1 = xyz(__ldg(r + 1)), n2 = xyz(__ldg(r + 2));
   float3 nm = interp_normal(h.u, h.v, n0, n1, n2);
   float ndl = ddot(nm, a.sh.l);
   float sigma = 0.0f;
@@ -306,9 +362,9 @@ __device__ __forceinline__ float3 shade(const RenderArgs& a, const Hit& h) {
   float k = a.sh.ka + a.sh.kd * sigma;
   float3 alb;
   if (a.tex) {
-    alb = tex_albedo(a, tex_coords(a, make_int3(i0, i1, i2), h.u, h.v));
+    alb = tex_albedo(a, tex_coords(a, __ldg(r + 7), __ldg(r + 8), h.u, h.v));
   } else {
-    float3 a0 = ld3(a.albedo + 3 * i0), a1 = ld3(a.albedo + 3 * i1), a2 = ld3(a.albedo + 3 * i2);
+    const float3 a0 = xyz(__ldg(r + 3)), a1 = xyz(__ldg(r + 4)), a2 = xyz(__ldg(r + 5));
     alb = make_float3(w * a0.x + h.u * a1.x + h.v * a2.x, w * a0.y + h.u * a1.y + h.v * a2.y,
                       w * a0.z + h.u * a1.z + h.v * a2.z);
   }
@@ -346,6 +402,7 @@ __device__ __forceinline__ RenderArgs for_inst(RenderArgs a, int inst) {
   a.tris += (size_t)inst * 3 * a.node_stride;
   a.verts += (size_t)inst * 3 * a.V;
   a.normals += (size_t)inst * 3 * a.V;
+  a.frec += (size_t)inst * kFaceRec * a.node_stride;
   return a;
 }
 
@@ -353,6 +410,16 @@ __device__ __forceinline__ RenderArgs for_inst(RenderArgs a, int inst) {
 __device__ __forceinline__ bool inst_active(const RenderArgs& a, int inst) {
   return !a.active || __ldg(&a.active[inst]) != 0;
 }
+
+__device__ __forceinline__ void write_face_records(const RenderArgs& a) {
+  const int F = a.max_visits - 1;
+  const long long n = (long long)a.n_inst * F;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const int inst = (int)(i / F);
+    if (inst_active(a, inst)) write_face_record(for_inst(a, inst), (int)(i - (long long)inst * F));
+  }
+}
+__global__ void k_face_records(RenderArgs a) { write_face_records(a); }
 
 // work-item region of an instance
 __device__ __forceinline__ int inst_ibase(const RenderArgs& a, int inst) { return a.vt ? a.it[inst].ibase : 0; }
@@ -570,9 +637,27 @@ struct GatherSmem {        // per warp
   float4 pl[5];
 };
 
+// screen positions of a triangle's corners and how far (in pixels, x and y) its edges
+// are moved outward by a pixel test that must keep every pixel a sample can hit it in;
+// not positive: no such test (the box alone)
+struct ScreenTri {
+  float x[3], y[3];
+  float margin;
+};
+
 // screen box (padded by half a pixel; unbounded if a vertex is not in front of the
 // camera) and nearest camera depth of triangle record k
-__device__ __forceinline__ void project_record(const RenderArgs& a, const Cam& cam, int k, float4& bb, float& zmin) {
+//
+// The margin: a sample the float32 intersection accepts lies within the rounding of
+// that test and of this projection from the triangle.  Both are a few float32 steps
+// (2^-24) of the camera distance in pixels; the test's part grows by the edges'
+// foreshortening, at most |edge| in pixels over the triangle's height on the screen.
+// 32 steps of a generous distance plus 1/16 pixel covers them many times over; where
+// that exceeds half a pixel (slivers, extreme cameras), or is not a number, the box,
+// which is padded by half a pixel, decides alone.
+template <bool TRI = false>
+__device__ __forceinline__ void project_record(const RenderArgs& a, const Cam& cam, int k, float4& bb, float& zmin,
+                                               ScreenTri* st = nullptr) {
   float4 t0 = __ldg(&a.tris[3 * k]), t1 = __ldg(&a.tris[3 * k + 1]), t2 = __ldg(&a.tris[3 * k + 2]);
   float3 v[3] = {make_float3(t0.x, t0.y, t0.z), make_float3(t0.x + t0.w, t0.y + t1.x, t0.z + t1.y),
                  make_float3(t0.x + t1.z, t0.y + t1.w, t0.z + t2.x)};
@@ -592,6 +677,27 @@ __device__ __forceinline__ void project_record(const RenderArgs& a, const Cam& c
     bx1 = fmaxf(bx1, sx);
     by0 = fminf(by0, sy);
     by1 = fmaxf(by1, sy);
+    if (TRI) {
+      st->x[m] = sx;
+      st->y[m] = sy;
+    }
+  }
+  if (TRI) {
+    const float dx1 = st->x[1] - st->x[0], dy1 = st->y[1] - st->y[0];
+    const float dx2 = st->x[2] - st->x[0], dy2 = st->y[2] - st->y[0];
+    const float area = fabsf(dx1 * dy2 - dx2 * dy1);
+    const float longest = fmaxf(fmaxf(fabsf(dx1) + fabsf(dy1), fabsf(dx2) + fabsf(dy2)),
+                                fabsf(dx2 - dx1) + fabsf(dy2 - dy1));
+    const float focal = fabsf(cam.fx) + fabsf(cam.fy);
+    const float edge = fabsf(t0.w) + fabsf(t1.x) + fabsf(t1.y) + fabsf(t1.z) + fabsf(t1.w) + fabsf(t2.x);
+    const float dist = fabsf(v[0].x) + fabsf(v[0].y) + fabsf(v[0].z) + edge + fabsf(cam.t[0]) + fabsf(cam.t[1]) +
+                       fabsf(cam.t[2]) + fabsf(cam.c[0]) + fabsf(cam.c[1]) + fabsf(cam.c[2]);
+    const float screen = fabsf(bx0) + fabsf(bx1) + fabsf(by0) + fabsf(by1) + fabsf(cam.cx) + fabsf(cam.cy);
+    const float px = focal / zmin;
+    const float grow = 1.0f + edge * px * longest / area;
+    const float m = 0.0625f + 1.9073486e-6f * (px * dist * grow + screen);
+    // the height test keeps the orientation's sign, and so the edges' sides, certain
+    st->margin = front && m <= 0.5f && area > m * longest ? m : 0.0f;
   }
   if (front) {
     bb = make_float4(bx0 - 0.5f, by0 - 0.5f, bx1 + 0.5f, by1 + 0.5f);
@@ -756,161 +862,216 @@ __device__ __forceinline__ unsigned warp_transpose32(unsigned x) {
   return x;
 }
 
-// closest hits of a lane's S rays (same origin, all in pixel (x0 + lane % 8,
-// y0 + lane / 8)) among the K pool candidates at `off`, which are sorted by nearest
-// depth.  The warp loads the candidates 32 at a time, one per lane (depth, screen box
-// and triangle record in three coalesced loads); each lane tests its candidate's box
-// against the sub-tile's 32 pixel squares, and a bit transpose gives every lane the
-// candidates that can hold a sample of its own pixel.  Each lane then walks only
-// those, in depth order, taking their records by shuffles from the lanes that loaded
-// them, so the lanes of one iteration each test a different candidate instead of
-// idling while the warp steps through candidates that miss their pixel.  A lane stops
-// at the first candidate nearer than none of its rays' hits (the list is depth-sorted,
-// so no later one is nearer).  Every ray tests the same candidates in the same order
-// as a scan of the whole list would, so each gets exactly the hit the one-ray search
-// gives it.  `live[j]` rays take part.
-template <bool STATS, int S>
-__device__ __forceinline__ void closest_candidates(const RenderArgs& a, int off, int K, int x0, int y0,
-                                                   const bool (&live)[S], const float (&sx)[S], const float (&sy)[S],
-                                                   float3 o, const float3 (&d)[S], Hit (&h)[S], Counts& cnt) {
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  bool done = true;
+// bits of box_pixel_mask's pixels that also meet the triangle moved outward by its
+// margin: for each edge the pixel's corner farthest inside decides, so with E = A x +
+// B y + C >= 0 inside, pixel (c, r) stays when A c + B r + C' >= 0, C' the edge's value
+// at the sub-tile's first pixel plus that corner's and the margin's share; every row's
+// columns are then an interval
+__device__ __forceinline__ unsigned tri_pixel_mask(float4 b, const ScreenTri& t, int x0, int y0) {
+  unsigned mask = box_pixel_mask(b, x0, y0);
+  if (!(t.margin > 0.0f) || !mask) return mask;
+  float px[3], py[3];
 #pragma unroll
-  for (int j = 0; j < S; ++j) {
-    h[j] = Hit{-1, INFINITY, 0.0f, 0.0f};
-    done = done && !live[j];
+  for (int k = 0; k < 3; ++k) {
+    px[k] = t.x[k] - (float)x0;
+    py[k] = t.y[k] - (float)y0;
   }
-  for (int c0 = 0; c0 < K; c0 += 32) {
-    if (!__any_sync(full, !done)) break;
-    // this block of candidates, one per lane; a pool index out of range ends the scan
-    const int cl = c0 + lane;
-    const bool have = cl < K;
-    const bool ok = have && in_range(a.status, off + cl, 0, a.wk.pool_cap);
-    float zl = 0.0f;
-    float4 bl = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    int kl = 0;
-    if (ok) {
-      zl = __ldg(&a.wk.z[off + cl]);
-      bl = __ldg(&a.wk.bb[off + cl]);
-      kl = __ldg(&a.wk.rec[off + cl]);
-    }
-    const unsigned bad = __ballot_sync(full, have && !ok);
-    int n = min(32, K - c0);
-    if (bad) n = min(n, __ffs(bad) - 1);
-    unsigned pm = 0u;
-    if (lane < n) {
-      pm = box_pixel_mask(bl, x0, y0);
-      if (STATS) ++cnt.cands;
-    }
-    unsigned m = warp_transpose32(pm);   // bit i: candidate c0 + i meets this lane's pixel
-    if (done) m = 0u;
-    for (;;) {
-      const bool act = m != 0u;
-      if (!__any_sync(full, act)) break;
-      const int i = act ? __ffs(m) - 1 : 0;
-      m &= m - 1u;
-      const float zm = __shfl_sync(full, zl, i);
-      const float bx0 = __shfl_sync(full, bl.x, i), by0 = __shfl_sync(full, bl.y, i);
-      const float bx1 = __shfl_sync(full, bl.z, i), by1 = __shfl_sync(full, bl.w, i);
-      const int k = __shfl_sync(full, kl, i);
-      if (!act) continue;
-      const float zlim = zm - (1e-4f * fabsf(zm) + 1e-6f);
-      bool want[S];
-      bool any = false;
+  const float area = (px[1] - px[0]) * (py[2] - py[0]) - (px[2] - px[0]) * (py[1] - py[0]);
+  const float sg = area < 0.0f ? -1.0f : 1.0f;
+  float lo[4] = {0.0f, 0.0f, 0.0f, 0.0f}, hi[4] = {7.0f, 7.0f, 7.0f, 7.0f};
 #pragma unroll
-      for (int j = 0; j < S; ++j) {
-        want[j] = live[j] && !(h[j].t < zlim);
-        any = any || want[j];
-      }
-      if (!any) {   // no later candidate is nearer either
-        done = true;
-        m = 0u;
-        continue;
-      }
-      bool inside = false;
+  for (int k = 0; k < 3; ++k) {
+    const int q = (k + 1) % 3;
+    const float A = sg * (py[k] - py[q]), B = sg * (px[q] - px[k]);
+    const float C = -(A * px[k] + B * py[k]) + t.margin * (fabsf(A) + fabsf(B)) + fmaxf(A, 0.0f) + fmaxf(B, 0.0f);
+    const float inv = 1.0f / fmaxf(fabsf(A), 1e-20f);
 #pragma unroll
-      for (int j = 0; j < S; ++j) {
-        if (STATS && want[j]) ++cnt.cands;
-        want[j] = want[j] && sx[j] >= bx0 && sx[j] <= bx1 && sy[j] >= by0 && sy[j] <= by1;
-        inside = inside || want[j];
-      }
-      if (!inside) continue;
-      if (!in_range(a.status, k, 0, a.max_visits - 1)) continue;
+    for (int r = 0; r < 4; ++r) {
+      const float c = (B * (float)r + C) * inv;   // columns c' >= -c (A >= 0) or c' <= c
+      if (A >= 0.0f) lo[r] = fmaxf(lo[r], -c);
+      else hi[r] = fminf(hi[r], c);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int c0 = (int)fminf(ceilf(lo[r]), 8.0f), c1 = (int)fmaxf(floorf(hi[r]), -1.0f);
+    const unsigned cols = c0 <= c1 ? (0xffu >> (7 - c1)) & (0xffu << c0) : 0u;
+    mask &= (cols << (8 * r)) | ~(0xffu << (8 * r));
+  }
+  return mask;
+}
+
+// A warp's candidates in shared memory: what the intersection of a primary ray with
+// each needs.  Primary rays start at the camera centre o, so of Moller-Trumbore's
+// s = o - v0, q = s x e1 and e2 . q only depend on the candidate; they are computed
+// once (the same operations, so the same float32 values) instead of once per ray.
+// Arrays of float4: lanes reading neighbouring candidates meet no bank conflict.
+constexpr int kCandCap = 48;
+struct CandTile {
+  float4 e1[kCandCap];   // e1, depth below which no ray's hit lets the candidate matter
+  float4 e2[kCandCap];   // e2, triangle id
+  float4 s[kCandCap];    // s, e2 . q
+  float4 q[kCandCap];    // q
+};
+
+// candidates [c0, c0 + n), n <= 32, of the list at `off` into slots slot0 .. (one per
+// lane); returns the lane's pixel's candidates, bit i = slot slot0 + i
+template <bool STATS>
+__device__ __forceinline__ unsigned stage_candidates(const RenderArgs& a, CandTile& ct, int slot0, int off, int c0, int n,
+                                                     float3 o, Counts& cnt) {
+  const int lane = threadIdx.x & 31;
+  unsigned pm = 0u;
+  if (lane < n) {
+    const int i = off + c0 + lane;
+    const float z = __ldg(&a.wk.z[i]);
+    const int k = __ldg(&a.wk.rec[i]);
+    pm = __ldg(&a.wk.pm[i]);
+    if (STATS) ++cnt.cands;
+    if (pm && in_range(a.status, k, 0, a.max_visits - 1)) {
       const float4 ta = __ldg(&a.tris[3 * k]), tb = __ldg(&a.tris[3 * k + 1]), tc = __ldg(&a.tris[3 * k + 2]);
-      const float3 v0 = make_float3(ta.x, ta.y, ta.z), e1 = make_float3(ta.w, tb.x, tb.y),
-                   e2 = make_float3(tb.z, tb.w, tc.x);
-      const int id = __float_as_int(tc.y);
-#pragma unroll
-      for (int j = 0; j < S; ++j) {
-        if (!want[j]) continue;
-        if (STATS) ++cnt.tris;
-        float t, u, v;
-        if (mt_hit(o, d[j], v0, e1, e2, t, u, v) && (t < h[j].t || (t == h[j].t && id < h[j].tri))) {
-          h[j].tri = id;
-          h[j].t = t;
-          h[j].u = u;
-          h[j].v = v;
-        }
-      }
+      const float3 e1 = make_float3(ta.w, tb.x, tb.y), e2 = make_float3(tb.z, tb.w, tc.x);
+      const float3 s = dsub(o, xyz(ta)), q = dcross(s, e1);
+      if (!in_range(a.status, __float_as_int(tc.y), 0, a.max_visits - 1)) pm = 0u;
+      ct.e1[slot0 + lane] = make_float4(e1.x, e1.y, e1.z, z - (1e-4f * fabsf(z) + 1e-6f));
+      ct.e2[slot0 + lane] = make_float4(e2.x, e2.y, e2.z, tc.y);
+      ct.s[slot0 + lane] = make_float4(s.x, s.y, s.z, ddot(e2, q));
+      ct.q[slot0 + lane] = make_float4(q.x, q.y, q.z, 0.0f);
+    } else {
+      pm = 0u;
     }
-    if (bad) break;
+  }
+  __syncwarp();
+  return warp_transpose32(pm);
+}
+
+// Walk of the candidates in m (bit i = slot slot0 + i, in depth order) by a lane's S
+// rays: the float32 Moller-Trumbore test and closest-hit rule of mt_hit / trace, with
+// the candidate's part taken from the tile.  u, v >= 0 and u + v <= 1 imply u <= 1, and
+// det = 0 makes u infinite or not a number, which fails the test, so both of mt_hit's
+// checks are kept; 1 / det is the correctly rounded reciprocal in both.  A lane stops at
+// the first candidate nearer than none of its hits (the list is depth-sorted).  Rays
+// that take no part start with t = -1, nearer than any hit.
+template <bool STATS, int S>
+__device__ __forceinline__ void walk_candidates(const CandTile& ct, int slot0, unsigned m, const float3 (&d)[S],
+                                                Hit (&h)[S], bool& done, Counts& cnt) {
+  while (m) {
+    const int i = slot0 + __ffs(m) - 1;
+    m &= m - 1u;
+    const float4 c1 = ct.e1[i];
+    float tmax = h[0].t;
+#pragma unroll
+    for (int j = 1; j < S; ++j) tmax = fmaxf(tmax, h[j].t);
+    if (tmax < c1.w) {
+      done = true;
+      break;
+    }
+    const float4 c2 = ct.e2[i], c3 = ct.s[i], c4 = ct.q[i];
+    const float3 e1 = xyz(c1), e2 = xyz(c2), s = xyz(c3), q = xyz(c4);
+    const int id = __float_as_int(c2.w);
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+      if (STATS && h[j].t >= 0.0f) ++cnt.tris;
+      const float3 p = dcross(d[j], e2);
+      const float inv = __frcp_rn(ddot(e1, p));
+      const float u = __fmul_rn(ddot(s, p), inv);
+      const float v = __fmul_rn(ddot(d[j], q), inv);
+      const float t = __fmul_rn(c3.w, inv);
+      if (fminf(u, v) >= 0.0f && __fadd_rn(u, v) <= 1.0f && t > 0.0f &&
+          (t < h[j].t || (t == h[j].t && id < h[j].tri)))
+        h[j] = Hit{id, t, u, v};
+    }
   }
 }
 
-// Radiance sums of samples [s0, s1) of this lane's pixel (all lanes call it), traced
-// S at a time (the tuning's rays per lane); the radiance is added in sample order.
-template <bool STATS, int S, bool TRACE = true>
-__device__ __forceinline__ void shade_samples(const RenderArgs& a, const SubTile& t, const Cam& cam, int off, int K,
-                                              int s0, int s1, float3& acc, int& misses, Counts& cnt) {
-  const int lane = threadIdx.x & 31;
-  const int px = t.x0 + (lane % kSubW), py = t.y0 + (lane / kSubW);
-  const bool valid = px < t.W && py < t.H;
+// what a warp keeps of the sub-tile it works on
+struct WarpTile {
+  CandTile cand;
+  SubTile t;
+  Cam cam;
+};
+
+// sub-tile t and its first kCandCap candidates into the warp's tile (all lanes call);
+// m0, m1: the lane's pixel's candidates in slots 0-31 and 32-63
+template <bool STATS>
+__device__ __forceinline__ void stage_tile(const RenderArgs& a, WarpTile& wt, const SubTile& t, int off, int K, unsigned& m0,
+                                           unsigned& m1, Counts& cnt) {
+  __syncwarp();   // every lane is done with the sub-tile before
+  if ((threadIdx.x & 31) == 0) wt.t = t;
+  const Cam& cam = warp_cam(&wt.cam, a.cams, t.view);
+  m0 = m1 = 0u;
+  if (K <= 0 || K > kCandCap) return;
   const float3 o = make_float3(cam.c[0], cam.c[1], cam.c[2]);
-  for (int sb = s0; sb < s1; sb += S) {
-    bool live[S];
-    float sx[S], sy[S];
-    float3 d[S];
-    Hit h[S];
+  m0 = stage_candidates<STATS>(a, wt.cand, 0, off, 0, min(K, 32), o, cnt);
+  if (K > 32) m1 = stage_candidates<STATS>(a, wt.cand, 32, off, 32, K - 32, o, cnt);
+}
+
+// closest hits of S rays of this lane's pixel among the K candidates at `off` (all
+// lanes call; `in`: the lane takes part).  Lists of up to kCandCap are in the tile
+// (m0, m1 from stage_tile); longer ones go through it in windows.
+template <bool STATS, int S>
+__device__ __forceinline__ void closest_staged(const RenderArgs& a, WarpTile& wt, int off, int K, unsigned m0, unsigned m1,
+                                               bool in, const float3 (&d)[S], Hit (&h)[S], Counts& cnt) {
+#pragma unroll
+  for (int j = 0; j < S; ++j) h[j] = Hit{-1, in ? INFINITY : -1.0f, 0.0f, 0.0f};
+  bool done = !in;
+  if (K <= kCandCap) {
+    if (!done) walk_candidates<STATS, S>(wt.cand, 0, m0, d, h, done, cnt);
+    if (!done) walk_candidates<STATS, S>(wt.cand, 32, m1, d, h, done, cnt);
+    __syncwarp();
+    return;
+  }
+  const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
+  for (int w = 0; w < K; w += 32) {
+    if (!__any_sync(0xffffffffu, !done)) break;
+    m0 = stage_candidates<STATS>(a, wt.cand, 0, off, w, min(32, K - w), o, cnt);
+    if (!done) walk_candidates<STATS, S>(wt.cand, 0, m0, d, h, done, cnt);
+    __syncwarp();   // every lane is done with the window
+  }
+}
+
+// Radiance of samples [s0, s0 + S) of this lane's pixel, traced together (all lanes
+// call it); added to the sums in sample order.
+template <bool STATS, int S, bool TRACE = true>
+__device__ __forceinline__ void shade_samples(const RenderArgs& a, WarpTile& wt, int off, int K, unsigned m0, unsigned m1,
+                                              int s0, float3& acc, int& misses, Counts& cnt) {
+  const int lane = threadIdx.x & 31;
+  const int px = wt.t.x0 + (lane % kSubW), py = wt.t.y0 + (lane / kSubW);
+  const bool valid = px < wt.t.W && py < wt.t.H;
+  float3 d[S];
+  Hit h[S];
+#pragma unroll
+  for (int j = 0; j < S; ++j) {
+    float u1, u2;
+    jitter(a, wt.t.ctr1, wt.t.W, px, py, s0 + j, u1, u2);
+    d[j] = primary_dir(wt.cam, __fadd_rn((float)px, u1), __fadd_rn((float)py, u2));
+    if (STATS && valid) {
+      ++cnt.samples;
+      ++cnt.rays;
+    }
+  }
+  if (K > 0) {
+    closest_staged<STATS, S>(a, wt, off, K, m0, m1, valid, d, h, cnt);
+  } else {
+    const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
 #pragma unroll
     for (int j = 0; j < S; ++j) {
-      live[j] = valid && sb + j < s1;
-      sx[j] = sy[j] = 0.0f;
-      if (live[j]) {
-        float u1, u2;
-        jitter(a, t.ctr1, t.W, px, py, sb + j, u1, u2);
-        sx[j] = __fadd_rn((float)px, u1);
-        sy[j] = __fadd_rn((float)py, u2);
-        if (STATS) {
-          ++cnt.samples;
-          ++cnt.rays;
-        }
-      }
-      d[j] = primary_dir(cam, sx[j], sy[j]);
+      h[j] = Hit{-1, INFINITY, 0.0f, 0.0f};
+      // K < 0: no usable candidate list, per-ray traversal (only the overflow kernel
+      // meets such sub-tiles; the shaders are built without it)
+      if (TRACE && valid) h[j] = trace<STATS>(a.nodes, a.tris, o, d[j], a.status, cnt, a.max_visits);
     }
-    if (K > 0) {
-      closest_candidates<STATS, S>(a, off, K, t.x0, t.y0, live, sx, sy, o, d, h, cnt);
+  }
+#pragma unroll
+  for (int j = 0; j < S; ++j) {
+    if (!valid) continue;
+    if (h[j].tri >= 0) {
+      if (STATS) ++cnt.hits;
+      float3 f = shade(a, h[j]);
+      acc.x += f.x;
+      acc.y += f.y;
+      acc.z += f.z;
     } else {
-#pragma unroll
-      for (int j = 0; j < S; ++j) {
-        h[j] = Hit{-1, INFINITY, 0.0f, 0.0f};
-        // K < 0: no usable candidate list, per-ray traversal (only the overflow kernel
-        // meets such sub-tiles; the shaders are built without it)
-        if (TRACE && live[j]) h[j] = trace<STATS>(a.nodes, a.tris, o, d[j], a.status, cnt, a.max_visits);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      if (!(valid && sb + j < s1)) continue;
-      if (h[j].tri >= 0) {
-        if (STATS) ++cnt.hits;
-        float3 f = shade(a, h[j]);
-        acc.x += f.x;
-        acc.y += f.y;
-        acc.z += f.z;
-      } else {
-        ++misses;
-      }
+      ++misses;
     }
   }
 }
@@ -931,215 +1092,269 @@ __device__ __forceinline__ void write_pixel(const RenderArgs& a, const SubTile& 
   image[3 * pix + 2] = acc.z * inv_spp + bgc.z * fm;
 }
 
-// dL/dverts (through u, v at the fixed ray) and dL/dnormals of one shaded hit with
-// upstream g = dL/df: dv[0..8] = dL/d(v0, v1, v2), dn[0..8] = dL/d(n0, n1, n2)
-struct HitGrad {
-  float dv[9], dn[9];
+// Where a backward's vertex sums go: vertex i's dL/dv and dL/dn, added with atomics
+// whose result is not read.  Float sums lie as [V][8] (dv, 0, dn, 0), so that a vertex
+// takes two 16-byte reductions instead of six of four bytes; float64 and fixed-point
+// sums as [V][3] then [V][3].
+struct SumF32 {
+  float* p;
+  __device__ __forceinline__ void add(int V, int i, float3 dv, float3 dn) const {
+    float* q = p + 8 * (size_t)i;
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(dv.x), "f"(dv.y), "f"(dv.z), "f"(0.0f)
+                 : "memory");
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q + 4), "f"(dn.x), "f"(dn.y), "f"(dn.z), "f"(0.0f)
+                 : "memory");
+  }
+};
+template <class T>
+struct SumWide {   // double, or unsigned long long (fixed point)
+  T* p;
+  __device__ __forceinline__ void add(int V, int i, float3 dv, float3 dn) const {
+    add3(p, i, dv.x, dv.y, dv.z);
+    add3(p + 3 * V, i, dn.x, dn.y, dn.z);
+  }
 };
 
-__device__ __forceinline__ void hit_grad(const RenderArgs& a, const Hit& h, const int3 f, float3 d,
-                                         float3 g, HitGrad& out) {
-  float3 n0 = ld3(a.normals + 3 * f.x), n1 = ld3(a.normals + 3 * f.y), n2 = ld3(a.normals + 3 * f.z);
-  float3 a0 = ld3(a.albedo + 3 * f.x), a1 = ld3(a.albedo + 3 * f.y), a2 = ld3(a.albedo + 3 * f.z);
-  const float u = h.u, v = h.v, w = 1.0f - u - v;
-  float3 nm = interp_normal(u, v, n0, n1, n2);
-  bool lit = ddot(nm, a.sh.l) > 0.0f;
-  float inv_len = rsqrtf(dot3(nm, nm));
-  float3 nh = make_float3(nm.x * inv_len, nm.y * inv_len, nm.z * inv_len);
-  float sigma = lit ? dot3(nh, a.sh.l) : 0.0f;
-  float k = a.sh.ka + a.sh.kd * sigma;
-  float3 dalb = make_float3(g.x * a.sh.lrgb.x * k, g.y * a.sh.lrgb.y * k, g.z * a.sh.lrgb.z * k);
-  float gu, gv;
-  float3 alb;
-  if (a.tex) {
-    // albedo = bilinear(texture, uv(u, v)): texel gradients, and the uv chain to (u, v)
-    const TexSample ts = tex_coords(a, f, u, v);
-    alb = tex_albedo(a, ts);
-    const float3 t00 = tex_texel(a, ts.i0, ts.j0), t10 = tex_texel(a, ts.i1, ts.j0);
-    const float3 t01 = tex_texel(a, ts.i0, ts.j1), t11 = tex_texel(a, ts.i1, ts.j1);
-    const float gx = 1.0f - ts.fx, gy = 1.0f - ts.fy;
-    const float dax = (gy * (t10.x - t00.x) + ts.fy * (t11.x - t01.x)) * dalb.x +
-                      (gy * (t10.y - t00.y) + ts.fy * (t11.y - t01.y)) * dalb.y +
-                      (gy * (t10.z - t00.z) + ts.fy * (t11.z - t01.z)) * dalb.z;
-    const float day = (gx * (t01.x - t00.x) + ts.fx * (t11.x - t10.x)) * dalb.x +
-                      (gx * (t01.y - t00.y) + ts.fx * (t11.y - t10.y)) * dalb.y +
-                      (gx * (t01.z - t00.z) + ts.fx * (t11.z - t10.z)) * dalb.z;
-    const float dux = dax * (float)a.tex_w, duy = day * (float)a.tex_h;   // dL/d(uv of the hit)
-    const float2 q0 = __ldg(reinterpret_cast<const float2*>(a.uv) + f.x);
-    const float2 q1 = __ldg(reinterpret_cast<const float2*>(a.uv) + f.y);
-    const float2 q2 = __ldg(reinterpret_cast<const float2*>(a.uv) + f.z);
-    gu = dux * (q1.x - q0.x) + duy * (q1.y - q0.y);
-    gv = dux * (q2.x - q0.x) + duy * (q2.y - q0.y);
-    if (a.d_tex) {
-      const float wts[4] = {gx * gy, ts.fx * gy, gx * ts.fy, ts.fx * ts.fy};
-      const int ii[4] = {ts.i0, ts.i1, ts.i0, ts.i1}, jj[4] = {ts.j0, ts.j0, ts.j1, ts.j1};
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        add3(a.d_tex, jj[q] * a.tex_w + ii[q], wts[q] * dalb.x, wts[q] * dalb.y, wts[q] * dalb.z);
-    }
-  } else {
-    gu = dalb.x * (a1.x - a0.x) + dalb.y * (a1.y - a0.y) + dalb.z * (a1.z - a0.z);
-    gv = dalb.x * (a2.x - a0.x) + dalb.y * (a2.y - a0.y) + dalb.z * (a2.z - a0.z);
-    alb = make_float3(w * a0.x + u * a1.x + v * a2.x, w * a0.y + u * a1.y + v * a2.y, w * a0.z + u * a1.z + v * a2.z);
-  }
-  float3 dnm = make_float3(0.0f, 0.0f, 0.0f);
-  if (lit) {
-    float dsig = a.sh.kd * (g.x * alb.x * a.sh.lrgb.x + g.y * alb.y * a.sh.lrgb.y + g.z * alb.z * a.sh.lrgb.z);
-    float3 dnh = make_float3(dsig * a.sh.l.x, dsig * a.sh.l.y, dsig * a.sh.l.z);
-    float pr = dot3(nh, dnh);
-    dnm = make_float3((dnh.x - nh.x * pr) * inv_len, (dnh.y - nh.y * pr) * inv_len, (dnh.z - nh.z * pr) * inv_len);
-    gu += dnm.x * (n1.x - n0.x) + dnm.y * (n1.y - n0.y) + dnm.z * (n1.z - n0.z);
-    gv += dnm.x * (n2.x - n0.x) + dnm.y * (n2.y - n0.y) + dnm.z * (n2.z - n0.z);
-  }
-  out.dn[0] = w * dnm.x; out.dn[1] = w * dnm.y; out.dn[2] = w * dnm.z;
-  out.dn[3] = u * dnm.x; out.dn[4] = u * dnm.y; out.dn[5] = u * dnm.z;
-  out.dn[6] = v * dnm.x; out.dn[7] = v * dnm.y; out.dn[8] = v * dnm.z;
-  // barycentrics at the fixed ray: moving vertex k by dp moves the hit's (u, v, t)
-  // by -M^-1 (w_k dp) with M = [e1, e2, -d] and weights (w, u, v), so
-  // dL/dp_k = -w_k (gu (d x e2) + gv (e1 x d)) / D, D = e1 . (d x e2) -- written with
-  // the triangle's edges and the ray direction only (the camera-to-triangle offset,
-  // ~1000x an edge, cancels out of the algebra and would cost float32 digits)
-  float3 p0 = ld3(a.verts + 3 * f.x), p1 = ld3(a.verts + 3 * f.y), p2 = ld3(a.verts + 3 * f.z);
-  float3 e1 = make_float3(p1.x - p0.x, p1.y - p0.y, p1.z - p0.z);
-  float3 e2 = make_float3(p2.x - p0.x, p2.y - p0.y, p2.z - p0.z);
-  float3 dxe2 = cross3(d, e2), e1xd = cross3(e1, d);
-  float invD = 1.0f / dot3(e1, dxe2);
-  float q[3] = {(gu * dxe2.x + gv * e1xd.x) * invD, (gu * dxe2.y + gv * e1xd.y) * invD,
-                (gu * dxe2.z + gv * e1xd.z) * invD};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    out.dv[c] = -w * q[c];
-    out.dv[3 + c] = -u * q[c];
-    out.dv[6 + c] = -v * q[c];
-  }
-}
 
-template <class T>
-__device__ __forceinline__ void flush_tri(int3 f, const HitGrad& acc, T* dV, T* dN) {
-  add3(dV, f.x, acc.dv[0], acc.dv[1], acc.dv[2]);
-  add3(dV, f.y, acc.dv[3], acc.dv[4], acc.dv[5]);
-  add3(dV, f.z, acc.dv[6], acc.dv[7], acc.dv[8]);
-  add3(dN, f.x, acc.dn[0], acc.dn[1], acc.dn[2]);
-  add3(dN, f.y, acc.dn[3], acc.dn[4], acc.dn[5]);
-  add3(dN, f.z, acc.dn[6], acc.dn[7], acc.dn[8]);
+// Value arithmetic of the backward, every contraction spelled out: a window's sums are
+// the same in every kernel that differentiates it (HR_DETERMINISTIC relies on it).
+__device__ __forceinline__ float3 sub3(float3 a, float3 b) {
+  return make_float3(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y), __fsub_rn(a.z, b.z));
 }
+__device__ __forceinline__ float vdot(float3 a, float3 b) {
+  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
+__device__ __forceinline__ void addmul(float& s, float a, float b) { s = __fmaf_rn(a, b, s); }
+__device__ __forceinline__ void addmul(float3& s, float a, float3 b) {
+  addmul(s.x, a, b.x);
+  addmul(s.y, a, b.y);
+  addmul(s.z, a, b.z);
+}
+// a x + b y (+ c z)
+__device__ __forceinline__ float3 comb(float a, float3 x, float b, float3 y) {
+  return make_float3(__fmaf_rn(a, x.x, __fmul_rn(b, y.x)), __fmaf_rn(a, x.y, __fmul_rn(b, y.y)),
+                     __fmaf_rn(a, x.z, __fmul_rn(b, y.z)));
+}
+__device__ __forceinline__ float lerp_rn(float a, float b, float t) { return __fmaf_rn(t, __fsub_rn(b, a), a); }
 
-// End-of-item flush by the whole warp: lanes whose run is on a triangle no other
-// lane holds add their sums directly; lanes sharing a triangle (the usual case in a
-// coherent 8x4 sub-tile) are summed by a warp butterfly first and one lane adds the
-// group's sums, so the shared-memory atomics do not collide on the same addresses.
-template <class T>
-__device__ __forceinline__ void flush_tri_warp(int cur, int3 cf, const HitGrad& acc, T* dV, T* dN) {
-  const unsigned full = 0xffffffffu;
+// Samples whose hits are differentiated together.  Within a window a lane's hits are
+// taken triangle by triangle, whatever their order among the samples: the triangle's
+// record is read and its sums are added to memory once per window instead of once per
+// run of consecutive hits (64 random samples of a pixel that shows three triangles
+// change triangle two times out of three).
+constexpr int kGradWin = 16;
+struct GradTile {
+  WarpTile w;
+  float4 hit[kGradWin][32];   // (triangle, u, v, -); with a texture then (cell, fx, fy, k)
+};
+
+// Differentiation of one window (any lanes), samples s0 ..: `pend` = those of this lane
+// with a hit in gt.hit, G = upstream gradient x light colour.
+//
+// At a fixed ray, moving corner k by dp moves the hit's (u, v, t) by -M^-1 (w_k dp) with
+// M = [e1, e2, -d] and weights w = (1 - u - v, u, v), so
+//   dL/dp_k = -w_k (gu (d x e2) + gv (e1 x d)) / (e1 . (d x e2)),
+// which does not depend on d's length: with d = -s + u e1 + v e2 (s = centre - v0) it is
+//   dL/dp_k = -w_k (gu A + gv B + (gu u + gv v) N) / D,
+//   A = e2 x s, B = s x e1, N = e1 x e2, D = s . N,
+// vectors of the triangle alone.  So per triangle only the nine sums of w_k gu, w_k gv
+// and w_k (gu u + gv v) are kept, and no ray direction.  The albedo enters through its
+// dot products with G.
+//
+// Their float32 errors are common to all of a triangle's samples, and seen nearly
+// edge-on they are small differences of large products (and the gradient is large): a
+// triangle whose |cos| to the view is below kGrazing takes the first form, with each
+// sample's own direction (made again) and so its own rounding.
+constexpr float kGrazing = 1.0f / 32;
+template <bool STATS, class Sum>
+__device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, unsigned pend, int s0, float3 G, Sum sum,
+                                            Counts& cnt) {
   const int lane = threadIdx.x & 31;
-  const unsigned grp = __match_any_sync(full, cur);
-  const bool shared = __popc(grp) > 1;
-  if (cur >= 0 && !shared) flush_tri(cf, acc, dV, dN);
-  unsigned pending = __ballot_sync(full, cur >= 0 && shared && lane == __ffs(grp) - 1);
-  while (pending) {
-    const int leader = __ffs(pending) - 1;
-    pending &= pending - 1;
-    const int key = __shfl_sync(full, cur, leader);
-    const bool in = cur == key;
-    HitGrad sum;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-      float x = in ? acc.dv[c] : 0.0f, y = in ? acc.dn[c] : 0.0f;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        x += __shfl_xor_sync(full, x, o);
-        y += __shfl_xor_sync(full, y, o);
-      }
-      sum.dv[c] = x;
-      sum.dn[c] = y;
+  const unsigned all = pend;
+  const float3 o = make_float3(gt.w.cam.c[0], gt.w.cam.c[1], gt.w.cam.c[2]);
+  while (pend) {
+    const int tri = __float_as_int(gt.hit[__ffs(pend) - 1][lane].x);
+    const float4* rec = a.frec + (size_t)kFaceRec * tri;
+    const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2), r3 = __ldg(rec + 3), r4 = __ldg(rec + 4),
+                 r5 = __ldg(rec + 5), r6 = __ldg(rec + 6), r8 = __ldg(rec + 8);
+    // this triangle's samples
+    unsigned m = 0u;
+    for (unsigned q = pend; q; q &= q - 1u) {
+      const int j = __ffs(q) - 1;
+      if (__float_as_int(gt.hit[j][lane].x) == tri) m |= 1u << j;
     }
-    if (lane == leader) flush_tri(cf, sum, dV, dN);
-  }
-}
-
-// Gradient of samples [s0, s1) of this lane's pixel (upstream g, `live` lanes only;
-// all lanes call it), traced S at a time and differentiated in sample order; added to
-// dV [V][3] / dN [V][3] per run of hits on one triangle.
-template <bool STATS, int S, class T, bool TRACE = true>
-__device__ __forceinline__ void grad_samples(const RenderArgs& a, const SubTile& t, const Cam& cam, int off, int K,
-                                             int s0, int s1, bool live, float3 g, T* dV, T* dN, Counts& cnt) {
-  const int lane = threadIdx.x & 31;
-  const int px = t.x0 + (lane % kSubW), py = t.y0 + (lane / kSubW);
-  const float3 o = make_float3(cam.c[0], cam.c[1], cam.c[2]);
-  int cur = -1;
-  int3 cf = make_int3(0, 0, 0);
-  HitGrad acc;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) acc.dv[c] = acc.dn[c] = 0.0f;
-  for (int sb = s0; sb < s1; sb += S) {
-    bool lv[S];
-    float sx[S], sy[S];
-    float3 d[S];
-    Hit h[S];
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      lv[j] = live && sb + j < s1;
-      sx[j] = sy[j] = 0.0f;
-      if (lv[j]) {
-        float u1, u2;
-        jitter(a, t.ctr1, t.W, px, py, sb + j, u1, u2);
-        sx[j] = __fadd_rn((float)px, u1);
-        sy[j] = __fadd_rn((float)py, u2);
-        if (STATS) {
-          ++cnt.samples;
-          ++cnt.rays;
-        }
-      }
-      d[j] = primary_dir(cam, sx[j], sy[j]);
-    }
-    if (K > 0) {
-      closest_candidates<STATS, S>(a, off, K, t.x0, t.y0, lv, sx, sy, o, d, h, cnt);
-    } else {
-#pragma unroll
-      for (int j = 0; j < S; ++j) {
-        h[j] = Hit{-1, INFINITY, 0.0f, 0.0f};
-        if (TRACE && lv[j]) h[j] = trace<STATS>(a.nodes, a.tris, o, d[j], a.status, cnt, a.max_visits);
-      }
-    }
-    // one copy of the differentiation for the S rays (the trace above is unrolled for
-    // its independent loads; unrolling this too multiplies the kernel's largest body
-    // S times and the warps then wait on instruction fetch): ray j is picked by
-    // selects, which keeps h and d in registers
-#pragma unroll 1
-    for (int j = 0; j < S; ++j) {
-      bool lj = lv[0];
-      Hit hj = h[0];
-      float3 dj = d[0];
-#pragma unroll
-      for (int q = 1; q < S; ++q)
-        if (j == q) {
-          lj = lv[q];
-          hj = h[q];
-          dj = d[q];
-        }
-      if (!lj || hj.tri < 0) continue;
+    pend &= ~m;
+    const float3 n0 = xyz(r0), n1 = xyz(r1), n2 = xyz(r2);
+    const float c0 = vdot(G, xyz(r3)), cu = vdot(G, sub3(xyz(r4), xyz(r3))), cv = vdot(G, sub3(xyz(r5), xyz(r3)));
+    float4 t01 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.tex) t01 = __ldg(rec + 7);
+    const float3 e1 = make_float3(r3.w, r4.w, r5.w), e2 = xyz(r6);
+    const float3 s = dsub(o, make_float3(r6.w, r8.z, r8.w)), nn = dcross(e1, e2);
+    const float D = vdot(s, nn);
+    const bool grazing = __fmul_rn(D, D) < __fmul_rn(kGrazing * kGrazing, __fmul_rn(vdot(s, s), vdot(nn, nn)));
+    // grazing: the sums of w_k q, q = (gu (d x e2) + gv (e1 x d)) / (e1 . (d x e2)),
+    // component by component
+    float su[3] = {0.f, 0.f, 0.f}, sv[3] = {0.f, 0.f, 0.f}, sn[3] = {0.f, 0.f, 0.f};
+    float3 dn[3] = {make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f), make_float3(0.f, 0.f, 0.f)};
+    while (m) {
+      const int j = __ffs(m) - 1;
+      m &= m - 1u;
+      const float4 hj = gt.hit[j][lane];
       if (STATS) ++cnt.hits;
-      if (hj.tri != cur) {
-        if (cur >= 0) {
-          flush_tri(cf, acc, dV, dN);
-#pragma unroll
-          for (int c = 0; c < 9; ++c) acc.dv[c] = acc.dn[c] = 0.0f;
-        }
-        cur = hj.tri;
-        cf = make_int3(__ldg(&a.faces[3 * cur]), __ldg(&a.faces[3 * cur + 1]), __ldg(&a.faces[3 * cur + 2]));
+      const float u = hj.y, v = hj.z, w[3] = {__fsub_rn(__fsub_rn(1.0f, u), v), u, v};
+      const float3 nm = interp_normal(u, v, n0, n1, n2);
+      const bool lit = ddot(nm, a.sh.l) > 0.0f;
+      const float inv_len = rsqrtf(vdot(nm, nm));
+      const float3 nh = make_float3(__fmul_rn(nm.x, inv_len), __fmul_rn(nm.y, inv_len), __fmul_rn(nm.z, inv_len));
+      const float sigma = lit ? vdot(nh, a.sh.l) : 0.0f;
+      const float k = __fmaf_rn(a.sh.kd, sigma, a.sh.ka);
+      float gu, gv, galb;   // dL/du, dL/dv through the albedo; G . albedo
+      if (a.tex) {
+        // albedo = bilinear(texture, uv(u, v)); its texel gradients are added below
+        const TexSample ts = tex_coords(a, t01, r8, u, v);
+        const float t00 = vdot(G, tex_texel(a, ts.i0, ts.j0)), t10 = vdot(G, tex_texel(a, ts.i1, ts.j0));
+        const float t0y = vdot(G, tex_texel(a, ts.i0, ts.j1)), t1y = vdot(G, tex_texel(a, ts.i1, ts.j1));
+        const float dx = lerp_rn(__fsub_rn(t10, t00), __fsub_rn(t1y, t0y), ts.fy);
+        const float dy = lerp_rn(__fsub_rn(t0y, t00), __fsub_rn(t1y, t10), ts.fx);
+        const float dux = __fmul_rn(__fmul_rn(dx, k), (float)a.tex_w), duy = __fmul_rn(__fmul_rn(dy, k), (float)a.tex_h);
+        gu = __fmaf_rn(dux, __fsub_rn(t01.z, t01.x), __fmul_rn(duy, __fsub_rn(t01.w, t01.y)));
+        gv = __fmaf_rn(dux, __fsub_rn(r8.x, t01.x), __fmul_rn(duy, __fsub_rn(r8.y, t01.y)));
+        galb = lerp_rn(lerp_rn(t00, t10, ts.fx), lerp_rn(t0y, t1y, ts.fx), ts.fy);
+        if (a.d_tex) gt.hit[j][lane] = make_float4(__int_as_float(ts.cell), ts.fx, ts.fy, k);
+      } else {
+        gu = __fmul_rn(k, cu);
+        gv = __fmul_rn(k, cv);
+        galb = __fmaf_rn(v, cv, __fmaf_rn(u, cu, c0));
       }
-      HitGrad hg;
-      hit_grad(a, hj, cf, dj, g, hg);
-      // rounded adds: no contraction with the products inside hit_grad, so a run's sum
-      // is the same in every kernel that traces it
+      if (lit) {
+        // through the normal: dL/dn of the interpolated n = kd galb (l - nh (nh . l)) / |n|
+        const float f = __fmul_rn(__fmul_rn(a.sh.kd, galb), inv_len);
+        const float3 dnm = make_float3(__fmul_rn(f, __fmaf_rn(-nh.x, sigma, a.sh.l.x)), __fmul_rn(f, __fmaf_rn(-nh.y, sigma, a.sh.l.y)),
+                                       __fmul_rn(f, __fmaf_rn(-nh.z, sigma, a.sh.l.z)));
+        gu = __fadd_rn(gu, vdot(dnm, sub3(n1, n0)));
+        gv = __fadd_rn(gv, vdot(dnm, sub3(n2, n0)));
 #pragma unroll
-      for (int c = 0; c < 9; ++c) {
-        acc.dv[c] = __fadd_rn(acc.dv[c], hg.dv[c]);
-        acc.dn[c] = __fadd_rn(acc.dn[c], hg.dn[c]);
+        for (int q = 0; q < 3; ++q) addmul(dn[q], w[q], dnm);
+      }
+      float gn = __fmaf_rn(gu, u, __fmul_rn(gv, v));
+      if (grazing) {
+        const WarpTile& wt = gt.w;
+        const int px = wt.t.x0 + (lane % kSubW), py = wt.t.y0 + (lane / kSubW);
+        float u1, u2;
+        jitter(a, wt.t.ctr1, wt.t.W, px, py, s0 + j, u1, u2);
+        const float3 d = primary_dir(wt.cam, __fadd_rn((float)px, u1), __fadd_rn((float)py, u2));
+        const float3 dxe2 = dcross(d, e2), e1xd = dcross(e1, d), q = comb(gu, dxe2, gv, e1xd);
+        const float invD = 1.0f / vdot(e1, dxe2);
+        gu = __fmul_rn(q.x, invD);
+        gv = __fmul_rn(q.y, invD);
+        gn = __fmul_rn(q.z, invD);
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        addmul(su[q], w[q], gu);
+        addmul(sv[q], w[q], gv);
+        addmul(sn[q], w[q], gn);
       }
     }
+    float3 A = dcross(e2, s), B = dcross(s, e1), N = nn;
+    float inv = -1.0f / D;
+    if (grazing) {
+      A = make_float3(1.f, 0.f, 0.f);
+      B = make_float3(0.f, 1.f, 0.f);
+      N = make_float3(0.f, 0.f, 1.f);
+      inv = -1.0f;
+    }
+    const int iv[3] = {__float_as_int(r0.w), __float_as_int(r1.w), __float_as_int(r2.w)};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      float3 dv = comb(__fmul_rn(su[k], inv), A, __fmul_rn(sv[k], inv), B);
+      addmul(dv, __fmul_rn(sn[k], inv), N);
+      sum.add(a.V, iv[k], dv, dn[k]);
+    }
   }
-  flush_tri_warp(cur, cf, acc, dV, dN);
+  if (!a.d_tex) return;
+  // texel gradients, cell by cell: the four corners' sums of weight x k, times G
+  for (pend = all; pend;) {
+    const int cell = __float_as_int(gt.hit[__ffs(pend) - 1][lane].x);
+    float wt[4] = {0.f, 0.f, 0.f, 0.f};
+    for (unsigned q = pend; q; q &= q - 1u) {
+      const int j = __ffs(q) - 1;
+      const float4 hj = gt.hit[j][lane];
+      if (__float_as_int(hj.x) != cell) continue;
+      pend &= ~(1u << j);
+      const float ky = hj.w * hj.z, k0 = hj.w - ky;
+      wt[1] += k0 * hj.y;
+      wt[0] += k0 - k0 * hj.y;
+      wt[3] += ky * hj.y;
+      wt[2] += ky - ky * hj.y;
+    }
+    TexSample ts;
+    ts.cell = cell;
+    tex_corners(a, ts);
+    const int ii[4] = {ts.i0, ts.i1, ts.i0, ts.i1}, jj[4] = {ts.j0, ts.j0, ts.j1, ts.j1};
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      add3(a.d_tex, jj[q] * a.tex_w + ii[q], wt[q] * G.x, wt[q] * G.y, wt[q] * G.z);
+  }
+}
+
+// hits of samples [s0, s0 + S) of this lane's pixel into window entries j0 .. (all lanes
+// call it; `live` lanes take part); returns the lane's entries with a hit
+template <bool STATS, int S, bool TRACE>
+__device__ __forceinline__ unsigned trace_samples(const RenderArgs& a, GradTile& gt, int off, int K, unsigned m0, unsigned m1,
+                                                  int s0, int j0, bool live, Counts& cnt) {
+  const int lane = threadIdx.x & 31;
+  const WarpTile& wt = gt.w;
+  const int px = wt.t.x0 + (lane % kSubW), py = wt.t.y0 + (lane / kSubW);
+  float3 d[S];
+  Hit h[S];
+#pragma unroll
+  for (int j = 0; j < S; ++j) {
+    float u1, u2;
+    jitter(a, wt.t.ctr1, wt.t.W, px, py, s0 + j, u1, u2);
+    d[j] = primary_dir(wt.cam, __fadd_rn((float)px, u1), __fadd_rn((float)py, u2));
+    if (STATS && live) {
+      ++cnt.samples;
+      ++cnt.rays;
+    }
+  }
+  if (K > 0) {
+    closest_staged<STATS, S>(a, gt.w, off, K, m0, m1, live, d, h, cnt);
+  } else {
+    const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+      h[j] = Hit{-1, INFINITY, 0.0f, 0.0f};
+      if (TRACE && live) h[j] = trace<STATS>(a.nodes, a.tris, o, d[j], a.status, cnt, a.max_visits);
+    }
+  }
+  unsigned hits = 0u;
+#pragma unroll
+  for (int j = 0; j < S; ++j) {
+    if (h[j].tri < 0) continue;
+    gt.hit[j0 + j][lane] = make_float4(__int_as_float(h[j].tri), h[j].u, h[j].v, 0.0f);
+    hits |= 1u << (j0 + j);
+  }
+  return hits;
+}
+
+// Gradient of samples [s0, s1) of this lane's pixel (upstream g, `live` lanes only; all
+// lanes call it after stage_tile), traced S at a time.  The windows and the order of a
+// window's sums depend on [s0, s1) alone.
+template <bool STATS, int S, class Sum, bool TRACE = true>
+__device__ __forceinline__ void grad_samples(const RenderArgs& a, GradTile& gt, int off, int K, unsigned m0, unsigned m1,
+                                             int s0, int s1, bool live, float3 g, Sum sum, Counts& cnt) {
+  const float3 G = make_float3(g.x * a.sh.lrgb.x, g.y * a.sh.lrgb.y, g.z * a.sh.lrgb.z);
+  for (int w0 = s0; w0 < s1; w0 += kGradWin) {
+    const int n = min(kGradWin, s1 - w0);
+    unsigned pend = 0u;
+    int j = 0;
+    for (; j + S <= n; j += S) pend |= trace_samples<STATS, S, TRACE>(a, gt, off, K, m0, m1, w0 + j, j, live, cnt);
+    if (S > 1)
+      for (; j < n; ++j) pend |= trace_samples<STATS, 1, TRACE>(a, gt, off, K, m0, m1, w0 + j, j, live, cnt);
+    grad_window<STATS>(a, gt, pend, w0, G, sum, cnt);
+    __syncwarp();
+  }
 }
 
 // this lane's upstream gradient dL/df / spp; `live` = non-zero adjoint
@@ -1208,8 +1423,8 @@ constexpr int kBinPairs = 8;   // (view, record) pairs per warp
 // one sub-tile of a pair's range: count it, or (FILL) write the record into the
 // sub-tile's pool range at the next free slot
 template <bool FILL>
-__device__ __forceinline__ void bin_visit(const RenderArgs& a, unsigned* __restrict__ bin, int s, int k, float zm,
-                                          float4 bb) {
+__device__ __forceinline__ void bin_visit(const RenderArgs& a, unsigned* __restrict__ bin, int s, int x0, int y0, int k,
+                                          float zm, float4 bb, const ScreenTri& tri) {
   if (!FILL) {
     atomicAdd(&bin[s], 1u);
     return;
@@ -1221,6 +1436,7 @@ __device__ __forceinline__ void bin_visit(const RenderArgs& a, unsigned* __restr
   a.wk.rec[pk.x + slot] = k;
   a.wk.z[pk.x + slot] = zm;
   a.wk.bb[pk.x + slot] = bb;
+  a.wk.pm[pk.x + slot] = tri_pixel_mask(bb, tri, x0, y0);
 }
 
 // Each warp takes kBinPairs consecutive pairs i = (active view i / F, record i % F),
@@ -1242,6 +1458,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin(RenderArgs a0, unsigned* __
     int st0 = 0, nsx = 1, k = 0, area = 0;
     float zm = 0.0f;
     float4 bb = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    ScreenTri tri{};
     BinRange r{0, -1, 0, -1};
     if (lane < kBinPairs && i < total) {
       const int g = visit_view(a0, (int)(i / F));
@@ -1252,7 +1469,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin(RenderArgs a0, unsigned* __
         const RenderArgs a = for_inst(a0, t.inst);
         const Cam cam = load_cam(a.cams, g);
         if (!record_behind(a, cam, k)) {
-          project_record(a, cam, k, bb, zm);
+          project_record<FILL>(a, cam, k, bb, zm, &tri);
           r = bin_range(bb, nsx, (t.H + kSubH - 1) / kSubH);
           if (r.c0 <= r.c1 && r.r0 <= r.r1) area = (r.c1 - r.c0 + 1) * (r.r1 - r.r0 + 1);
         }
@@ -1283,16 +1500,27 @@ __global__ void __launch_bounds__(kBinThreads) k_bin(RenderArgs a0, unsigned* __
       const int na = __shfl_sync(full, area, own);
       const float z = __shfl_sync(full, zm, own);
       float4 b = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      ScreenTri tv{};
       if (FILL) {
         b.x = __shfl_sync(full, bb.x, own);
         b.y = __shfl_sync(full, bb.y, own);
         b.z = __shfl_sync(full, bb.z, own);
         b.w = __shfl_sync(full, bb.w, own);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          tv.x[m] = __shfl_sync(full, tri.x[m], own);
+          tv.y[m] = __shfl_sync(full, tri.y[m], own);
+        }
+        tv.margin = __shfl_sync(full, tri.margin, own);
       }
       if (q >= T) continue;
       const int w = c1 - c0 + 1, local = q - (end - na);
-      bin_visit<FILL>(a0, bin, s0 + (r0 + local / w) * n + c0 + local % w, kk, z, b);
+      const int col = c0 + local % w, row = r0 + local / w;
+      bin_visit<FILL>(a0, bin, s0 + row * n + col, col * kSubW, row * kSubH, kk, z, b, tv);
     }
+  }
+  if (!FILL) {   // the shading records, for the shader three launches later
+    write_face_records(a0);
   }
 }
 
@@ -1481,6 +1709,7 @@ __global__ void __launch_bounds__(kGroupThreads) k_background(RenderArgs a0, flo
 // memory, the boxes then projected again from the records), written back in order
 struct SortSmem {   // per warp
   int leaf[kLeafCap];
+  unsigned pm[kLeafCap];
   float key[kLeafCap];
   int idx[kLeafCap];
 };
@@ -1502,10 +1731,12 @@ __global__ void __launch_bounds__(kRenderThreads) k_bin_sort(RenderArgs a0) {
       // sort of (depth, lane) across the warp; lane c then takes the c-th record's box
       // and index from its lane
       int k = 0;
+      unsigned pm = 0u;
       float4 bb = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       float key = INFINITY;
       if (lane < K) {
         k = a0.wk.rec[off + lane];
+        pm = a0.wk.pm[off + lane];
         key = a0.wk.z[off + lane];
         bb = a0.wk.bb[off + lane];
       }
@@ -1525,12 +1756,14 @@ __global__ void __launch_bounds__(kRenderThreads) k_bin_sort(RenderArgs a0) {
         }
       }
       const int kc = __shfl_sync(0xffffffffu, k, src);
+      const unsigned pc = __shfl_sync(0xffffffffu, pm, src);
       const float4 bc = make_float4(__shfl_sync(0xffffffffu, bb.x, src), __shfl_sync(0xffffffffu, bb.y, src),
                                     __shfl_sync(0xffffffffu, bb.z, src), __shfl_sync(0xffffffffu, bb.w, src));
       if (lane < K) {
         a0.wk.bb[off + lane] = bc;
         a0.wk.z[off + lane] = key;
         a0.wk.rec[off + lane] = kc;
+        a0.wk.pm[off + lane] = pc;
       }
       continue;
     }
@@ -1542,13 +1775,16 @@ __global__ void __launch_bounds__(kRenderThreads) k_bin_sort(RenderArgs a0) {
     while (P < K) P <<= 1;
     for (int j = lane; j < P; j += 32) {
       int k = 0;
+      unsigned pm = 0u;
       float z = INFINITY;
       if (j < K) {
         k = a.wk.rec[off + j];
+        pm = a.wk.pm[off + j];
         z = a.wk.z[off + j];
         if (!in_range(a.status, k, 0, a.max_visits - 1)) k = 0;
       }
       ss.leaf[j] = k;
+      ss.pm[j] = pm;
       ss.key[j] = z;
       ss.idx[j] = j;
     }
@@ -1582,6 +1818,7 @@ __global__ void __launch_bounds__(kRenderThreads) k_bin_sort(RenderArgs a0) {
       a.wk.bb[off + c] = bb;
       a.wk.z[off + c] = zm;
       a.wk.rec[off + c] = k;
+      a.wk.pm[off + c] = ss.pm[j];
     }
     __syncwarp();
   }
@@ -1682,6 +1919,7 @@ __global__ void __launch_bounds__(kRenderThreads) k_gather(RenderArgs a_in, cons
           a.wk.bb[off + c] = bb;
           a.wk.z[off + c] = zm;
           a.wk.rec[off + c] = k;
+          a.wk.pm[off + c] = box_pixel_mask(bb, t.x0, t.y0);
         }
       } else {
         // pool full: per-ray traversal for this sub-tile, with K's count kept as
@@ -1766,6 +2004,7 @@ __global__ void __launch_bounds__(kGroupThreads, 4) k_items_bwd(RenderArgs a0, c
     const bool heavy = need && heavy_item(a0, pk.y, C, t.spp);
     place_items(a0, need, st, t.inst, pk.y, C, heavy);
   }
+  write_face_records(a0);   // for the shader that follows
   flush_counts<STATS>(cnt, stats);
 }
 
@@ -1788,19 +2027,88 @@ __device__ __forceinline__ void item_samples(int c, int C, int spp, int& s0, int
   s1 = (int)((long long)(c + 1) * spp / C);
 }
 
-// fetch the next work item of instance `inst` (lane 0 takes it, the warp shares it);
-// -1 when the instance's region is exhausted
-__device__ __forceinline__ int next_item(const RenderArgs& a, int inst, int n) {
-  int it = 0;
-  if ((threadIdx.x & 31) == 0) it = (int)atomicAdd(&a.wk.ctr[3 + 2 * inst], 1u);
-  it = __shfl_sync(0xffffffffu, it, 0);
-  return it < n ? it : -1;
+// A warp's place in the work items.  Each instance's items are handed out from one
+// counter, in runs of `run` consecutive items (several per warp are left to balance the
+// load): consecutive items are mostly of one sub-tile, whose candidates the shaders
+// then stage once.  The next run is asked for when the last item of a run is handed
+// out, so the counter's round trip passes beside the shading.  The blocks of an SM
+// start on one instance (its triangles stay in the SM's L1) and the instances are
+// spread over the SMs; a warp whose instance has run out looks for one with items left,
+// 32 at a time.
+struct Cursor {
+  int inst;            // instance, -1 before the first
+  int n, nf, run;      // its items, front items and run length
+  int pos, end;        // the rest of the current run
+  int pre;             // lane 0: first item of the run asked for (valid when `asked`)
+  bool asked;
+};
+constexpr int kMaxRun = 16;
+
+__device__ __forceinline__ void enter_instance(const RenderArgs& a, Cursor& c, int inst) {
+  c.inst = inst;
+  c.n = item_count(a, inst);
+  c.nf = front_count(a, inst);
+  // about eight runs per warp if every warp had its share of the instances
+  const long long warps = max(1LL, (long long)gridDim.x * (blockDim.x / 32) / a.n_inst);
+  c.run = (int)min((long long)kMaxRun, max(1LL, c.n / (8 * warps)));
+  c.pos = c.end = 0;
+  c.asked = false;
 }
 
-// the sub-tile and candidate list of item `gi` (global index); false for a blanked or
-// corrupt item
-__device__ __forceinline__ bool load_item(const RenderArgs& a, int gi, int4& item, SubTile& t, int2& pk) {
-  item = a.wk.items[gi];
+__device__ __forceinline__ void ask_run(const RenderArgs& a, Cursor& c) {
+  if ((threadIdx.x & 31) == 0) c.pre = (int)atomicAdd(&a.wk.ctr[3 + 2 * c.inst], (unsigned)c.run);
+  c.asked = true;
+}
+
+__device__ __forceinline__ Cursor start_items(const RenderArgs& a) {
+  Cursor c;
+  c.pre = 0;
+  // the blocks an SM holds at once differ by the number of SMs
+  const int sms = max(1, a.num_sms), home = (int)((long long)(blockIdx.x % sms) * a.n_inst / sms);
+  enter_instance(a, c, home);
+  return c;
+}
+
+// the next item (region slot in `slot`, without the instance's base); false at the end
+__device__ __forceinline__ bool next_item(const RenderArgs& a, Cursor& c, int& slot) {
+  const unsigned full = 0xffffffffu;
+  for (;;) {
+    if (c.pos < c.end) {
+      slot = item_slot(a, c.inst, c.pos, c.nf);
+      if (++c.pos == c.end) ask_run(a, c);
+      return true;
+    }
+    if (c.n > 0) {
+      if (!c.asked) ask_run(a, c);
+      c.pos = __shfl_sync(full, c.pre, 0);
+      c.asked = false;
+      if (c.pos < c.n) {   // (a negative position could only come from a wrapped counter)
+        c.pos = max(c.pos, 0);
+        c.end = min(c.pos + c.run, c.n);
+        continue;
+      }
+      c.pos = c.end = 0;
+    }
+    int found = -1;
+    for (int base = 1; base < a.n_inst && found < 0; base += 32) {
+      const int k = base + (threadIdx.x & 31);
+      int inst = c.inst + k;
+      if (inst >= a.n_inst) inst -= a.n_inst;
+      bool left = false;
+      if (k < a.n_inst) {
+        const unsigned taken = *reinterpret_cast<volatile unsigned*>(&a.wk.ctr[3 + 2 * inst]);
+        left = taken < (unsigned)item_count(a, inst);
+      }
+      const unsigned b = __ballot_sync(full, left);
+      if (b) found = __shfl_sync(full, inst, __ffs(b) - 1);
+    }
+    if (found < 0) return false;
+    enter_instance(a, c, found);
+  }
+}
+
+// the sub-tile and candidate list of an item; false for a blanked or corrupt item
+__device__ __forceinline__ bool load_item(const RenderArgs& a, const int4& item, SubTile& t, int2& pk) {
   if (item.x < 0) return false;   // a blanked slot
   if (!in_range(a.status, item.x, 0, subtile_count(a))) return false;
   t = subtile(a, item.x);
@@ -1846,39 +2154,68 @@ __device__ __forceinline__ void finish_item(const RenderArgs& a, const SubTile& 
   if (lane == 0) a.wk.st_done[item.x] = 0u;   // ready for the next launch
 }
 
-// warps take work items, instance after instance; S samples per lane at a time
+// warps take work items; S samples per lane at a time.  The sub-tile's description, its
+// camera and its candidates are kept in the warp's shared memory from item to item.
+// Bound by instruction issue (52 % active, 20 of 32 lanes) with the latency of the
+// items' chains beside it.  Against a walk that took every candidate's box and record
+// through shuffles and global loads for each group of samples: 64 M -> 36 M warp
+// instructions and 112 -> 75 us on 8 x 512x384 at 16 spp; 64 hands, 612 views: 6.45 ->
+// 3.30 ms; 1024 views of 256^2 at 4 spp, whose items hold one sample: 2.52 -> 0.98 ms.
 template <bool STATS, int S>
-__global__ void __launch_bounds__(kRenderThreads, 6) k_shade_fwd(RenderArgs a_in, float* __restrict__ image,
-                                                                  unsigned long long* stats) {
+__global__ void __launch_bounds__(kRenderThreads, kFwdMinBlocks) k_shade_fwd(RenderArgs a_in, float* __restrict__ image,
+                                                                             unsigned long long* stats) {
   pdl_wait();
-  __shared__ Cam scam[kWarps];
+  __shared__ WarpTile tiles[kWarps];
+  WarpTile& wt = tiles[threadIdx.x >> 5];
   const RenderArgs a0 = with_iter(a_in);
   Counts cnt;
-  for (int inst = 0; inst < a0.n_inst; ++inst) {
-    const int n = item_count(a0, inst), nf = front_count(a0, inst), ibase = inst_ibase(a0, inst);
-    const RenderArgs a = for_inst(a0, inst);
-    for (;;) {
-      const int it = next_item(a, inst, n);
-      if (it < 0) break;
-      const int slot = ibase + item_slot(a, inst, it, nf);
-      int4 item;
+  Cursor cur = start_items(a0);
+  int at = -1, K = 0, off = 0, slot;   // the sub-tile staged
+  unsigned m0 = 0u, m1 = 0u;
+  while (next_item(a0, cur, slot)) {
+    const int gi = inst_ibase(a0, cur.inst) + slot;
+    const int4 item = a0.wk.items[gi];
+    if (item.x != at) {
       SubTile t;
       int2 pk;
-      if (!load_item(a, slot, item, t, pk) || t.inst != inst) continue;
+      at = -1;
+      if (!load_item(a0, item, t, pk) || t.inst != cur.inst) continue;
       if (pk.y < 0) continue;   // no candidate list: k_overflow traces this item
-      const Cam& cam = warp_cam(&scam[threadIdx.x >> 5], a.cams, t.view);
-      int s0, s1;
-      item_samples(item.y, item.z, t.spp, s0, s1);
-      float3 acc = make_float3(0.0f, 0.0f, 0.0f);
-      int misses = 0;
-      shade_samples<STATS, S, false>(a, t, cam, pk.x, pk.y, s0, s1, acc, misses, cnt);
-      finish_item(a, t, item, slot, acc, misses, image);
+      at = item.x;
+      off = pk.x;
+      K = pk.y;
+      const RenderArgs a = for_inst(a0, cur.inst);
+      stage_tile<STATS>(a, wt, t, off, K, m0, m1, cnt);
     }
+    const RenderArgs a = for_inst(a0, cur.inst);
+    int s0, s1;
+    item_samples(item.y, item.z, wt.t.spp, s0, s1);
+    float3 acc = make_float3(0.0f, 0.0f, 0.0f);
+    int misses = 0;
+    for (; s0 + S <= s1; s0 += S) shade_samples<STATS, S, false>(a, wt, off, K, m0, m1, s0, acc, misses, cnt);
+    if (S > 1)
+      for (; s0 < s1; ++s0) shade_samples<STATS, 1, false>(a, wt, off, K, m0, m1, s0, acc, misses, cnt);
+    finish_item(a, wt.t, item, gi, acc, misses, image);
   }
   flush_counts<STATS>(cnt, stats);
 }
 
-// one warp per sub-tile with items: its item sums in item order, then the pixel
+struct FwdTile {
+  WarpTile w;
+};
+template <bool STATS>
+__device__ __forceinline__ void overflow_grad(const RenderArgs& a, GradTile& gt, int inst, int off, int K, unsigned m0,
+                                              unsigned m1, int s0, int s1, bool live, float3 g, Counts& cnt) {
+  if (a.wk.det)
+    grad_samples<STATS, 1>(a, gt, off, K, m0, m1, s0, s1, live, g,
+                           SumWide<unsigned long long>{a.wk.fx + (size_t)inst * 6 * a.V}, cnt);
+  else
+    grad_samples<STATS, 1>(a, gt, off, K, m0, m1, s0, s1, live, g, SumF32{a.wk.extra + (size_t)inst * 8 * a.V}, cnt);
+}
+template <bool STATS>   // the forward overflow kernel never takes this branch
+__device__ __forceinline__ void overflow_grad(const RenderArgs&, FwdTile&, int, int, int, unsigned, unsigned, int, int, bool,
+                                              float3, Counts&) {}
+
 // The rare paths, kept out of the gather and the shaders so that their registers are
 // sized for their own work: (1) sub-tiles whose work items did not fit their
 // instance's region -- one warp does a whole sub-tile, all its samples, in the chunks
@@ -1890,6 +2227,10 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
                                                                                      const float* __restrict__ adjoint,
                                                             float* __restrict__ image, unsigned long long* stats) {
   pdl_wait();
+  typedef typename std::conditional<BWD, GradTile, FwdTile>::type Tile;
+  __shared__ Tile tiles[kWarps];
+  Tile& gt = tiles[threadIdx.x >> 5];
+  WarpTile& wt = gt.w;
   const RenderArgs a0 = with_iter(a_in);
   const int total = subtile_count(a0);
   const int n = (int)min(*reinterpret_cast<volatile unsigned*>(&a0.wk.ctr[2 + 2 * a0.n_inst]), (unsigned)total);
@@ -1904,26 +2245,24 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
     if (pk.y > 0 && !in_range(a.status, (long long)pk.x + pk.y - 1, 0, a.wk.pool_cap)) pk.y = -1;
     const Cam cam = load_cam(a.cams, t.view);
     if (BWD) {
-      // in the items' chunks too: each chunk's runs are added exactly as its work item
+      // in the items' chunks too: each chunk's sums are added exactly as its work item
       // would add them, so fixed-point sums do not depend on which sub-tiles overflowed
       bool live;
       const float3 g = lane_adjoint(a, t, adjoint, live);
       const int C = chunks_for(a, pk.y, t.spp);
+      unsigned m0, m1;
+      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, m1, cnt);
       for (int c = 0; c < C; ++c) {
         int s0, s1;
         item_samples(c, C, t.spp, s0, s1);
-        if (a.wk.det) {
-          unsigned long long* ex = a.wk.fx + (size_t)t.inst * 6 * a.V;
-          grad_samples<STATS, 1>(a, t, cam, pk.x, pk.y, s0, s1, live, g, ex, ex + 3 * a.V, cnt);
-        } else {
-          float* ex = a.wk.extra + (size_t)t.inst * 6 * a.V;
-          grad_samples<STATS, 1>(a, t, cam, pk.x, pk.y, s0, s1, live, g, ex, ex + 3 * a.V, cnt);
-        }
+        overflow_grad<STATS>(a, gt, t.inst, pk.x, pk.y, m0, m1, s0, s1, live, g, cnt);
       }
     } else {
       // the same chunks and the same order of sums as the work items and finish_item
       // would use, so a pixel's value does not depend on which path rendered it
       const int C = chunks_for(a, pk.y, t.spp);
+      unsigned m0, m1;
+      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, m1, cnt);
       float3 tot = make_float3(0.0f, 0.0f, 0.0f);
       float tmiss = 0.0f;
       for (int c = 0; c < C; ++c) {
@@ -1931,7 +2270,7 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
         item_samples(c, C, t.spp, s0, s1);
         float3 acc = make_float3(0.0f, 0.0f, 0.0f);
         int misses = 0;
-        shade_samples<STATS, 1>(a, t, cam, pk.x, pk.y, s0, s1, acc, misses, cnt);
+        for (; s0 < s1; ++s0) shade_samples<STATS, 1>(a, wt, pk.x, pk.y, m0, m1, s0, acc, misses, cnt);
         tot.x += acc.x;
         tot.y += acc.y;
         tot.z += acc.z;
@@ -1951,7 +2290,8 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
     int4 item;
     SubTile t;
     int2 pk;
-    if (!load_item(a0, slot, item, t, pk) || pk.y >= 0) continue;
+    item = a0.wk.items[slot];
+    if (!load_item(a0, item, t, pk) || pk.y >= 0) continue;
     const RenderArgs a = for_inst(a0, t.inst);
     const Cam cam = load_cam(a.cams, t.view);
     int s0, s1;
@@ -1959,17 +2299,15 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
     if (BWD) {
       bool live;
       const float3 g = lane_adjoint(a, t, adjoint, live);
-      if (a.wk.det) {
-        unsigned long long* ex = a.wk.fx + (size_t)t.inst * 6 * a.V;
-        grad_samples<STATS, 1>(a, t, cam, pk.x, pk.y, s0, s1, live, g, ex, ex + 3 * a.V, cnt);
-      } else {
-        float* ex = a.wk.extra + (size_t)t.inst * 6 * a.V;
-        grad_samples<STATS, 1>(a, t, cam, pk.x, pk.y, s0, s1, live, g, ex, ex + 3 * a.V, cnt);
-      }
+      unsigned m0, m1;
+      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, m1, cnt);
+      overflow_grad<STATS>(a, gt, t.inst, pk.x, pk.y, m0, m1, s0, s1, live, g, cnt);
     } else {
       float3 acc = make_float3(0.0f, 0.0f, 0.0f);
       int misses = 0;
-      shade_samples<STATS, 1>(a, t, cam, pk.x, pk.y, s0, s1, acc, misses, cnt);
+      unsigned m0, m1;
+      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, m1, cnt);
+      for (; s0 < s1; ++s0) shade_samples<STATS, 1>(a, wt, pk.x, pk.y, m0, m1, s0, acc, misses, cnt);
       finish_item(a, t, item, slot, acc, misses, image);
     }
   }
@@ -1980,15 +2318,19 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
 // every mode adds with atomic adds whose result is not read, which retire in L2
 // without holding up the warp (float adds to shared memory cost a read and a
 // compare-and-swap loop each, and made the sums a quarter of this kernel's time):
-//   kAccPartials  block b into partial b % nparts of `nparts` partials [6V]
+//   kAccPartials  block b into partial b % nparts of `nparts` partials [V][8]
 //                 (L2-resident, zeroed before the launch), summed in partial order by
 //                 k_reduce_partials (single instance)
 //   kAccDirect    every run of hits on one triangle straight into its instance's
-//                 extra [6V] (batches)
+//                 extra [V][8] (batches)
 //   kAccGlobal    meshes beyond kPartialMaxV vertices: into the instance's float64
 //                 extra64 [6V] (long runs of cancelling contributions)
 //   kAccFixed     HR_DETERMINISTIC: into the instance's fixed-point sums fx [6V]
 //                 (order-free integer atomics)
+// Bound by instruction issue and the latency of divergent loads.  With the hits of a
+// window differentiated triangle by triangle instead of run by run, the candidates from
+// the tile and vertices summed 16 bytes at a time: 64 hands, 612 views 7.4 -> 4.9 ms
+// (with the edge kernel beside it), textured 16 x 1024^2 at 64 spp 4.5 -> 3.0 ms.
 constexpr int kAccPartials = 0, kAccDirect = 1, kAccGlobal = 2, kAccFixed = 3;
 template <bool STATS, int ACC, int S>
 __global__ void __launch_bounds__(kRenderThreads, kBwdMinBlocks) k_shade_bwd(RenderArgs a_in,
@@ -1996,49 +2338,54 @@ __global__ void __launch_bounds__(kRenderThreads, kBwdMinBlocks) k_shade_bwd(Ren
                                                                              float* __restrict__ partials, int nparts,
                                                                              unsigned long long* stats) {
   pdl_wait();
-  __shared__ Cam scam[kWarps];
+  __shared__ GradTile tiles[kWarps];
+  GradTile& gt = tiles[threadIdx.x >> 5];
   const RenderArgs a0 = with_iter(a_in);
-  float* part = partials + (size_t)(blockIdx.x % nparts) * 6 * a0.V;
   Counts cnt;
-  for (int inst = 0; inst < a0.n_inst; ++inst) {
-    const int n = item_count(a0, inst), nf = front_count(a0, inst), ibase = inst_ibase(a0, inst);
+  Cursor cur = start_items(a0);
+  int at = -1, K = 0, off = 0, slot;   // the sub-tile staged
+  unsigned m0 = 0u, m1 = 0u;
+  bool live = false;
+  float3 g = make_float3(0.0f, 0.0f, 0.0f);
+  while (next_item(a0, cur, slot)) {
+    const int inst = cur.inst;
+    const int4 item = a0.wk.items[inst_ibase(a0, inst) + slot];
     const RenderArgs a = for_inst(a0, inst);
-    typedef typename std::conditional<
-        ACC == kAccGlobal, double, typename std::conditional<ACC == kAccFixed, unsigned long long, float>::type>::type
-        AccT;
-    AccT* sdV;
-    if constexpr (ACC == kAccGlobal)
-      sdV = a0.wk.extra64 + (size_t)inst * 6 * a0.V;
-    else if constexpr (ACC == kAccFixed)
-      sdV = a0.wk.fx + (size_t)inst * 6 * a0.V;
-    else if constexpr (ACC == kAccDirect)
-      sdV = a0.wk.extra + (size_t)inst * 6 * a0.V;
-    else
-      sdV = part;
-    AccT* sdN = sdV + 3 * a0.V;
-    for (;;) {
-      const int it = next_item(a, inst, n);
-      if (it < 0) break;
-      int4 item;
+    if (item.x != at) {
       SubTile t;
       int2 pk;
-      if (!load_item(a, ibase + item_slot(a, inst, it, nf), item, t, pk) || t.inst != inst) continue;
+      at = -1;
+      if (!load_item(a0, item, t, pk) || t.inst != inst) continue;
       if (pk.y < 0) continue;   // no candidate list: k_overflow traces this item
-      bool live;
-      const float3 g = lane_adjoint(a, t, adjoint, live);
-      const Cam& cam = warp_cam(&scam[threadIdx.x >> 5], a.cams, t.view);
-      int s0, s1;
-      item_samples(item.y, item.z, t.spp, s0, s1);
-      grad_samples<STATS, S, AccT, false>(a, t, cam, pk.x, pk.y, s0, s1, live, g, sdV, sdN, cnt);
+      at = item.x;
+      off = pk.x;
+      K = pk.y;
+      g = lane_adjoint(a, t, adjoint, live);
+      stage_tile<STATS>(a, gt.w, t, off, K, m0, m1, cnt);
     }
+    int s0, s1;
+    item_samples(item.y, item.z, gt.w.t.spp, s0, s1);
+    if constexpr (ACC == kAccGlobal)
+      grad_samples<STATS, S, SumWide<double>, false>(a, gt, off, K, m0, m1, s0, s1, live, g,
+                                                     SumWide<double>{a0.wk.extra64 + (size_t)inst * 6 * a0.V}, cnt);
+    else if constexpr (ACC == kAccFixed)
+      grad_samples<STATS, S, SumWide<unsigned long long>, false>(
+          a, gt, off, K, m0, m1, s0, s1, live, g, SumWide<unsigned long long>{a0.wk.fx + (size_t)inst * 6 * a0.V}, cnt);
+    else
+      grad_samples<STATS, S, SumF32, false>(
+          a, gt, off, K, m0, m1, s0, s1, live, g,
+          SumF32{ACC == kAccDirect ? a0.wk.extra + (size_t)inst * 8 * a0.V
+                                   : partials + (size_t)(blockIdx.x % nparts) * 8 * a0.V},
+          cnt);
   }
   flush_counts<STATS>(cnt, stats);
 }
 
-// d_verts[i] = extra[i] + sum_b partials[b][i] (i < 3V), dN[i-3V] likewise.  A block
-// covers 32 entries with 16 groups of threads: group g sums partials g, g + 16, ...
-// in order, then the 16 group sums are added in group order (a fixed order for every
-// call).  blockIdx.y selects the instance (a batch has no partials).
+// d_verts and dN from the sums: word i of the [V][8] float sums is the float extra plus
+// every partial's word (and the float64 or fixed-point sum).  A block covers 32 words
+// with 16 groups of threads: group g sums partials g, g + 16, ... in order, then the 16
+// group sums are added in group order (a fixed order for every call).  blockIdx.y
+// selects the instance (a batch has no partials).
 constexpr int kRedEntries = 32, kRedGroups = 16;
 __global__ void __launch_bounds__(kRedEntries * kRedGroups) k_reduce_partials(
     const float* __restrict__ partials, const float* __restrict__ extra_all, const double* __restrict__ extra64_all,
@@ -2049,22 +2396,23 @@ __global__ void __launch_bounds__(kRedEntries * kRedGroups) k_reduce_partials(
   const int j = threadIdx.x % kRedEntries, g = threadIdx.x / kRedEntries;
   const int i = blockIdx.x * kRedEntries + j;
   float acc = 0.0f;
-  if (i < 6 * V) {
+  if (i < 8 * V) {
 #pragma unroll 4
-    for (int b = g; b < nblocks; b += kRedGroups) acc += partials[(size_t)b * 6 * V + i];
+    for (int b = g; b < nblocks; b += kRedGroups) acc += partials[(size_t)b * 8 * V + i];
   }
   red[g][j] = acc;
   __syncthreads();
-  if (g != 0 || i >= 6 * V) return;
-  const float* extra = extra_all + (size_t)blockIdx.y * 6 * V;
+  const int v = i / 8, c = i % 8;
+  if (g != 0 || i >= 8 * V || (c & 3) == 3) return;
   float* d_verts = d_verts_all + (size_t)blockIdx.y * 3 * V;
   float* dN = dN_all + (size_t)blockIdx.y * 3 * V;
-  float tot = extra[i];
-  if (extra64_all) tot = (float)(extra64_all[(size_t)blockIdx.y * 6 * V + i] + (double)tot);
-  if (fx_all) tot += from_fixed(fx_all[(size_t)blockIdx.y * 6 * V + i]);
+  const size_t wide = (size_t)blockIdx.y * 6 * V + (c < 3 ? 3 * v + c : 3 * V + 3 * v + c - 4);
+  float tot = extra_all[(size_t)blockIdx.y * 8 * V + i];
+  if (extra64_all) tot = (float)(extra64_all[wide] + (double)tot);
+  if (fx_all) tot += from_fixed(fx_all[wide]);
   for (int q = 0; q < kRedGroups; ++q) tot += red[q][j];
-  if (i < 3 * V) d_verts[i] = tot;
-  else dN[i - 3 * V] = tot;
+  if (c < 3) d_verts[3 * v + c] = tot;
+  else dN[3 * v + c - 4] = tot;
 }
 
 // per view: silhouette flags in edge order, compacted by a block-wide scan.  In a
@@ -2441,6 +2789,7 @@ RenderArgs make_args(Context* ctx, const hr_model* m, const float* verts, const 
   a.faces = m->faces;
   a.normals = ctx->normals;
   a.albedo = m->albedo;
+  a.frec = ctx->face_rec;
   a.cams = cams;
   a.bg = bg;
   a.N = N;
@@ -2461,6 +2810,7 @@ RenderArgs make_args(Context* ctx, const hr_model* m, const float* verts, const 
   a.wk.bb = ctx->pool_bb;
   a.wk.z = ctx->pool_z;
   a.wk.rec = ctx->pool_rec;
+  a.wk.pm = ctx->pool_pm;
   a.wk.pool_cap = ctx->pool_cap;
   a.wk.st = ctx->st_info;
   a.wk.items = ctx->items;
@@ -2478,6 +2828,7 @@ RenderArgs make_args(Context* ctx, const hr_model* m, const float* verts, const 
   a.wk.fx = ctx->acc_fx;
   a.wk.det = (o->flags & HR_DETERMINISTIC) != 0;
   a.node_stride = ctx->lim.max_F;
+  a.num_sms = ctx->num_sms;
   a.cand_per_chunk = ctx->tune.cand_per_chunk;
   a.max_chunks = ctx->tune.max_chunks;
   a.uv = m->uv;
@@ -2626,7 +2977,7 @@ int launch_render_bwd(Context* ctx, const hr_model* m, const float* verts, const
     // candidates of the sub-tiles with a non-zero adjoint: the interior shader's work
     // items, and the edge rays' candidate lists
     if (cudaMemsetAsync(ctx->work_ctr, 0, ctr_words(ni) * sizeof(unsigned), s) != cudaSuccess ||
-        cudaMemsetAsync(ctx->extra, 0, sizeof(float) * 6 * V * ni, s) != cudaSuccess)
+        cudaMemsetAsync(ctx->extra, 0, sizeof(float) * 8 * V * ni, s) != cudaSuccess)
       return HR_ERR_CUDA;
     // the forward's candidate lists still describe this scene when it used the same
     // vertices, cameras and sizes after the last build
@@ -2644,6 +2995,8 @@ int launch_render_bwd(Context* ctx, const hr_model* m, const float* verts, const
       // its own lists from a frustum walk of the BVH: the boxes must be current
       const int rc = launch_bvh_lazy_refit(ctx, 1, s);
       if (rc != HR_OK) return rc;
+      k_face_records<<<ctx->num_sms, kGroupThreads, 0, s>>>(a);
+      HR_CHECK_LAUNCH();
       if (st)
         k_gather<true><<<ctx->num_sms * ctx->tune.blocks_per_sm, kRenderThreads, 0, s>>>(a, adjoint,
                                                                             ctx->stats + kStatsPer);
@@ -2670,7 +3023,7 @@ int launch_render_bwd(Context* ctx, const hr_model* m, const float* verts, const
     if (!det && cudaMemsetAsync(ctx->dedge, 0, sizeof(float) * 3 * V * ni, es) != cudaSuccess) return HR_ERR_CUDA;
   }
   const auto reduce = [&](int acc, int nparts) {
-    launch_pdl(k_reduce_partials, dim3((6 * V + kRedEntries - 1) / kRedEntries, ni), dim3(kRedEntries * kRedGroups), 0,
+    launch_pdl(k_reduce_partials, dim3((8 * V + kRedEntries - 1) / kRedEntries, ni), dim3(kRedEntries * kRedGroups), 0,
                s, (const float*)ctx->partials, (const float*)ctx->extra,
                (const double*)(acc == kAccGlobal ? ctx->extra64 : nullptr),
                (const unsigned long long*)(det ? ctx->acc_fx : nullptr), acc == kAccPartials ? nparts : 0, V, d_verts,
@@ -2698,7 +3051,7 @@ int launch_render_bwd(Context* ctx, const hr_model* m, const float* verts, const
     const int blocks = ctx->num_sms * ctx->tune.bwd_blocks_per_sm;
     const int nparts = ctx->num_sms;
     if (acc == kAccPartials &&
-        cudaMemsetAsync(ctx->partials, 0, sizeof(float) * 6 * V * (size_t)nparts, s) != cudaSuccess)
+        cudaMemsetAsync(ctx->partials, 0, sizeof(float) * 8 * V * (size_t)nparts, s) != cudaSuccess)
       return HR_ERR_CUDA;
     tm.begin(kTimeBwdShade);
     launch_pdl(kern, dim3(blocks), dim3(kRenderThreads), 0, s, a, adjoint, ctx->partials, nparts,
