@@ -18,107 +18,15 @@
 // Every mbarrier wait is bounded (about one second of device time); a wait that
 // runs out sets a status bit, the CTA stops issuing work, waits (bounded) for its own
 // copies in flight, frees its tensor memory and returns.
-#include <cuda.h>
-#include <cuda_bf16.h>
-
 #include <mutex>
 
-#include "hr_internal.h"
+#include "hr_tcgen05.cuh"
 
 namespace hr {
 
 namespace {
 
 constexpr int kBM = 128, kBK = 64, kStages = 3, kGemmThreads = 192;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// bounded wait for the phase of `parity` to complete; false when it ran out
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  for (;;) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (globaltimer() - t0 > 1000000000ull) return false;   // 1 s
-  }
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// tcgen05 shared-memory matrix descriptor: K-major operand tile whose rows are 128
-// bytes (64 bf16), 128-byte swizzle, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);          // start address
-  d |= (uint64_t)1 << 16;                          // leading byte offset (unused with swizzle)
-  d |= (uint64_t)(1024 >> 4) << 32;                // stride byte offset: 8 rows x 128 B
-  d |= (uint64_t)1 << 46;                          // descriptor version
-  d |= (uint64_t)2 << 61;                          // 128-byte swizzle
-  return d;
-}
-
-// instruction descriptor of kind::f16: bf16 x bf16 -> f32, both K-major, M x N
-__host__ __device__ constexpr uint32_t mma_idesc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 struct GemmArgs {
   int M, N, K;
@@ -148,7 +56,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_id(), lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
   const int kt0 = blockIdx.z * g.kt_per_split;
   const int kt_total = (g.K / kBK);
@@ -174,49 +82,52 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // producer
+    const bool leader = elect_one();
     int issued = 0;
     for (int kt = 0; kt < nkt; ++kt) {
       const int s = kt % kStages;
       if (kt >= kStages && !mbar_wait(smem_u32(&empty_bar[s]), ((kt / kStages) + 1) & 1)) {
-        set_status(g.status, kStatusTimeout);
+        if (lane == 0) set_status(g.status, kStatusTimeout);
         atomicExch(&abort_flag, 1);
         break;
       }
       if (*reinterpret_cast<volatile int*>(&abort_flag)) break;
       const uint32_t fb = smem_u32(&full_bar[s]);
-      mbar_expect_tx(fb, kABytes + kBBytes);
-      tma_load_2d(smem_u32(sA + s * kABytes), &tmA, (kt0 + kt) * kBK, m0, fb);
-      tma_load_2d(smem_u32(sB + s * kBBytes), &tmB, (kt0 + kt) * kBK, n0, fb);
+      if (leader) {
+        mbar_expect_tx(fb, kABytes + kBBytes);
+        tma_load_2d(smem_u32(sA + s * kABytes), &tmA, (kt0 + kt) * kBK, m0, fb);
+        tma_load_2d(smem_u32(sB + s * kBBytes), &tmB, (kt0 + kt) * kBK, n0, fb);
+      }
       ++issued;
     }
     // copies still in flight must land before the CTA may exit
     for (int kt = max(0, issued - kStages); kt < issued; ++kt)
       mbar_wait(smem_u32(&full_bar[kt % kStages]), (kt / kStages) & 1);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // MMA issuer
     constexpr uint32_t idesc = mma_idesc(kBM, BN);
+    const bool leader = elect_one();
+    const uint32_t a0 = desc_lo(smem_u32(sA)), b0 = desc_lo(smem_u32(sB));
     bool ok = true;
     for (int kt = 0; kt < nkt; ++kt) {
       const int s = kt % kStages;
       if (!mbar_wait(smem_u32(&full_bar[s]), (kt / kStages) & 1)) {
-        set_status(g.status, kStatusTimeout);
+        if (lane == 0) set_status(g.status, kStatusTimeout);
         atomicExch(&abort_flag, 1);
         ok = false;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a0 = smem_u32(sA + s * kABytes), b0 = smem_u32(sB + s * kBBytes);
-#pragma unroll
-      for (int k = 0; k < kBK / 16; ++k)
-        mma_bf16(tmem, sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), idesc, (kt > 0 || k > 0) ? 1u : 0u);
-      mma_commit(smem_u32(&empty_bar[s]));   // the stage is free once these MMAs have read it
+      if (leader) {
+        mma_step(tmem, a0 + s * (kABytes >> 4), b0 + s * (kBBytes >> 4), idesc, kt > 0);
+        mma_commit(smem_u32(&empty_bar[s]));   // the stage is free once these MMAs have read it
+      }
     }
-    if (ok && nkt > 0) mma_commit(smem_u32(&done_bar));
-    if (!ok || nkt == 0) {
-      // nothing (more) will be computed: release the epilogue
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&done_bar)) : "memory");
+    if (leader) {
+      if (ok && nkt > 0) mma_commit(smem_u32(&done_bar));
+      else mbar_arrive(smem_u32(&done_bar));   // nothing (more) will be computed: release the epilogue
     }
   } else if (warp >= 2) {
     // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 = tile rows
@@ -320,19 +231,6 @@ EncodeTiledFn encode_fn() {
   return g_encode;
 }
 
-// 2-D bf16 tensor map over rows x K (K contiguous, row pitch ld elements), box 64 x box_rows
-bool make_map(CUtensorMap* map, const void* ptr, int rows, int K, int ld, int box_rows) {
-  EncodeTiledFn enc = encode_fn();
-  if (!enc) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int BN>
 size_t gemm_smem() {
   return 1024 + (size_t)kStages * (kBM * kBK * 2 + BN * kBK * 2);
@@ -348,6 +246,18 @@ int launch_gemm_bn(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs&
 }
 
 }  // namespace
+
+bool tma_map(CUtensorMap* map, const void* ptr, long long rows, int cols, int ld, int box_rows) {
+  EncodeTiledFn enc = encode_fn();
+  if (!enc) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+  cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 int configure_gemm_kernels() {
   if (cudaFuncSetAttribute(k_gemm_bf16<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem<32>()) !=
@@ -369,7 +279,7 @@ int launch_gemm(const void* A, int lda, const void* Bm, int ldb, int M, int N, i
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(Bm)) & 15) return HR_ERR_ARG;
   const int BN = N <= 32 ? 32 : (N <= 64 ? 64 : 128);
   CUtensorMap ta, tb;
-  if (!make_map(&ta, A, M, K, lda, kBM) || !make_map(&tb, Bm, N, K, ldb, BN)) return HR_ERR_CUDA;
+  if (!tma_map(&ta, A, M, K, lda, kBM) || !tma_map(&tb, Bm, N, K, ldb, BN)) return HR_ERR_CUDA;
   const int kt_total = K / kBK;
   if (splits > kt_total) splits = kt_total;
   GemmArgs g;

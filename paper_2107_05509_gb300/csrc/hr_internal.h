@@ -64,6 +64,21 @@ int launch_gemm(const void* A, int lda, const void* B, int ldb, int M, int N, in
                 void* C, int ldc, int out_bf16, int splits, float* split_buf, int* status, cudaStream_t s);
 int configure_gemm_kernels();
 
+// the proposal network's 3x3 stride-2 convolutions and weight gradients (hr_conv.cu); all
+// bf16, NHWC: X [NV][Hin][Hin][Cin], Y and dPre [NV][Hin / 2][Hin / 2][Cout], W [Cout][Kp],
+// wT [Kp][Cout], Hin a power of two, Cin 8 .. 128 and Cout 32 .. 128 powers of two.
+// dgrad: dX with the ReLU mask of X (needs Cin >= 32, Cout >= 64).  part: scratch.
+int configure_conv_kernels();
+int launch_conv_fwd(const void* X, int NV, int Hin, int Cin, const void* W, int Kp, const float* bias, int Cout, void* Y,
+                    int* status, cudaStream_t s);
+int launch_conv_dgrad(const void* dPre, int NV, int Hin, int Cin, const void* wT, int Cout, const void* X, void* dX,
+                      int* status, cudaStream_t s);
+int launch_conv_wgrad(const void* X, int NV, int Hin, int Cin, int Kp, const void* dPre, int Cout, float* dW, float* db,
+                      float* part, size_t part_floats, int* status, cudaStream_t s);
+// dW [N][K] = dPre^T x, db = column sums of dPre; x [rows][K], dPre [rows][N]
+int launch_dense_wgrad(const void* x, long long rows, int K, const void* dPre, int N, float* dW, float* db, float* part,
+                       size_t part_floats, int* status, cudaStream_t s);
+
 // per-device properties of the render kernels (persistent grid)
 int render_grid(int device, int* blocks, int* threads, int* num_sms);
 int subtiles_for(int views, int W, int H);

@@ -1,0 +1,52 @@
+"""Kernels at the sizes where their division of the work changes: fewer tiles than
+SMs, one more than a multiple, odd counts."""
+import numpy as np
+import pytest
+
+from oracle import net as N
+from tests import test_gpu_net as TN
+from tests.gpu_common import require_gpu, torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B_():
+    require_gpu()
+    from paper_2107_05509_gb300 import binding
+    return binding
+
+
+def _net_run(B_, copies):
+    p, X, cams = TN._case(2, 2)
+    net = B_.Net(2 * copies, 2)
+    net.set_params(torch.as_tensor(p, device="cuda"))
+    Xt = torch.as_tensor(X.astype(np.float32), device="cuda").to(torch.bfloat16)
+    net.set_inputs_bf16(Xt.repeat(copies, 1, 1, 1))
+    out = torch.empty((2 * copies, 61), device="cuda")
+    net.forward(torch.as_tensor(np.concatenate([cams] * copies), device="cuda"), out)
+    d_out = np.random.default_rng(7).normal(size=(2, 61)).astype(np.float32)
+    net.backward(torch.as_tensor(np.concatenate([d_out] * copies), device="cuda"))
+    g = torch.empty(net.P, device="cuda")
+    net.get_params(grads=g)
+    assert net.status() == B_.HR_OK
+    return out.cpu().numpy(), g.cpu().numpy().astype(np.float64)
+
+
+@pytest.mark.parametrize("copies", [3, 9, 40])
+def test_convolutions_are_sums_over_their_images(B_, copies):
+    """The gathered convolutions on copies of the four images that the network's tests
+    check against the oracle: 12 images (most SMs idle), 36 (tiles and splits do not
+    divide evenly), 160 (rings and accumulators wrap, more images than SMs).  Outputs
+    equal the single case's bit for bit in every copy.  Gradients are sums of equal
+    addends: they are `copies` times the single ones up to float32 accumulation of at
+    most 655360 products in pieces of at most 4096 (256 steps of the tensor cores, each
+    2^-24 of the running sum, 1.5e-5 per piece, with some cancellation): 1e-4 of the
+    layer's largest."""
+    out1, g1 = _net_run(B_, 1)
+    out, g = _net_run(B_, copies)
+    assert (out.reshape(copies, 2, 61) == out1).all()
+    for name, (w, b, n_out, K) in N.offsets()[0].items():
+        for lo, hi in ((w, w + n_out * K), (b, b + n_out)):
+            err = np.abs(g[lo:hi] - copies * g1[lo:hi]).max()
+            assert err <= 1e-4 * copies * np.abs(g1[lo:hi]).max(), (name, err)
