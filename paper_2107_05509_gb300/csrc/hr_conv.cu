@@ -639,12 +639,6 @@ __global__ void __launch_bounds__(32 * kRedWarps) k_wgrad_reduce(const float* __
   }
 }
 
-int sm_count() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 152;
-  return std::max(n, 1);
-}
-
 int ilog2(int x) {
   int l = 0;
   while ((1 << l) < x) ++l;

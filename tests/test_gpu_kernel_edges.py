@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from oracle import net as N
+from tests import test_gpu_gemm as TG
 from tests import test_gpu_net as TN
 from tests.gpu_common import require_gpu, torch
 
@@ -50,3 +51,14 @@ def test_convolutions_are_sums_over_their_images(B_, copies):
         for lo, hi in ((w, w + n_out * K), (b, b + n_out)):
             err = np.abs(g[lo:hi] - copies * g1[lo:hi]).max()
             assert err <= 1e-4 * copies * np.abs(g1[lo:hi]).max(), (name, err)
+
+
+@pytest.mark.parametrize("M,N,K,relu,bf16", [
+    (2048, 2048, 1024, False, True),    # the smallest that takes pairs, whole tiles
+    (2049, 2303, 1088, True, True),     # ragged on both sides, rows of C at odd addresses
+    (16389, 200, 1024, False, False),   # one column of tiles, the last with 5 rows
+    (2000, 5003, 512, True, False),     # two rounds of tiles, a short reduction
+])
+def test_gemm_on_pairs(B_, M, N, K, relu, bf16):
+    """Tolerance: that of the small tiles' test (float32 accumulation of K products)."""
+    TG.test_gemm_matches_float64((B_, B_.Context(8, 8, 8, 1, 8, 8)), M, N, K, 1, relu, bf16)
