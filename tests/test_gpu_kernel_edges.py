@@ -1,12 +1,14 @@
 """Kernels at the sizes where their division of the work changes: fewer tiles than
 SMs, one more than a multiple, odd counts."""
+import dataclasses
+
 import numpy as np
 import pytest
 
 from oracle import net as N
 from tests import test_gpu_gemm as TG
 from tests import test_gpu_net as TN
-from tests.gpu_common import require_gpu, torch
+from tests.gpu_common import hand, require_gpu, torch
 
 pytestmark = pytest.mark.gpu
 
@@ -62,3 +64,48 @@ def test_convolutions_are_sums_over_their_images(B_, copies):
 def test_gemm_on_pairs(B_, M, N, K, relu, bf16):
     """Tolerance: that of the small tiles' test (float32 accumulation of K products)."""
     TG.test_gemm_matches_float64((B_, B_.Context(8, 8, 8, 1, 8, 8)), M, N, K, 1, relu, bf16)
+
+
+@pytest.mark.parametrize("F", [1, 2, 3, 33, 255, 257, 1024, 1025, 2048, 2049, 4097, 8193])
+def test_trees_reach_every_triangle(B_, F):
+    """Full builds and refits around the powers of two of the sort, one and two leaves
+    per thread, the largest merged build (2048), search builds beyond and the multi-block
+    one (8193): separate triangles on two layers of a grid, in random order, each hit by a
+    ray of its own at t = 9.  A refit keeps the tree for other positions."""
+    rng = np.random.default_rng(F)
+    n = (F + 1) // 2
+    side = int(np.ceil(np.sqrt(n)))
+    order = rng.permutation(F)
+
+    def soup(order):
+        cell, layer = order // 2, order % 2
+        c = np.stack([cell % side, cell // side, layer.astype(np.float64)], 1)
+        tri = np.array([[-0.2, -0.2, 0], [0.3, -0.1, 0], [-0.1, 0.3, 0]])
+        orig = c + np.where(layer == 1, 9.0, -9.0)[:, None] * [0, 0, 1]
+        dirs = np.where(layer == 1, -1.0, 1.0)[:, None] * [0, 0, 1]
+        return (c[:, None] + tri).reshape(-1, 3), orig, dirs
+
+    h = hand()
+    faces = np.arange(3 * F, dtype=np.int32).reshape(F, 3)
+    one = lambda a: np.repeat(a[:1], 3 * F, 0)
+    v, _, _ = soup(order)
+    model = B_.Model(dataclasses.replace(
+        h, v_template=v.astype(np.float32), shapedirs=one(h.shapedirs), weights=one(h.weights), faces=faces,
+        edges=faces[:, :2].copy(), edge_faces=np.stack([np.arange(F), np.full(F, -1)], 1).astype(np.int32),
+        vf_offsets=np.arange(3 * F + 1, dtype=np.int32), vf_faces=np.repeat(np.arange(F, dtype=np.int32), 3),
+        albedo=one(h.albedo), uv=None))
+    ctx = B_.Context(3 * F, F, F, 1, 8, 8)
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a, np.float32), device="cuda")
+    counter = torch.full((1,), 3, dtype=torch.int32, device="cuda")
+    for refit in (False, True):
+        v, orig, dirs = soup(rng.permutation(F) if refit else order)
+        if refit:
+            B_.hr_update_bvh(ctx, model, t(v), counter, 8)
+        else:
+            B_.hr_build_bvh(ctx, model, t(v))
+        tri = torch.empty(F, dtype=torch.int32, device="cuda")
+        tuv = torch.empty((F, 3), device="cuda")
+        B_.hr_trace(ctx, t(orig), t(dirs), tri, tuv)
+        assert (tri.cpu().numpy() == np.arange(F)).all()
+        assert np.abs(tuv.cpu().numpy()[:, 0] - 9.0).max() <= 1e-5
+    assert B_.hr_get_status(ctx) == B_.HR_OK
