@@ -109,3 +109,20 @@ def test_trees_reach_every_triangle(B_, F):
         assert (tri.cpu().numpy() == np.arange(F)).all()
         assert np.abs(tuv.cpu().numpy()[:, 0] - 9.0).max() <= 1e-5
     assert B_.hr_get_status(ctx) == B_.HR_OK
+
+
+@pytest.mark.parametrize("W,Wo", [(2, 1), (510, 85), (514, 257), (65536, 32768)])
+def test_resampling_by_whole_factors(B_, W, Wo):
+    """Segments of a row (one channel column to more than a block), more taps than a
+    chunk (factor 6) and the longest rows.  Means of f x f uniform values
+    to float32 accumulation (36 products with weights exact to 2^-24): 2e-6."""
+    f = W // Wo
+    rng = np.random.default_rng(W)
+    img = rng.random((2, 2 * f, W, 3), dtype=np.float32)
+    m = rng.integers(0, 255, (2, 2 * f, W)).astype(np.uint8)
+    out, mout = torch.empty((2, 2, Wo, 3), device="cuda"), torch.empty((2, 2, Wo), dtype=torch.uint8, device="cuda")
+    B_.hr_area_resample(torch.as_tensor(img, device="cuda"), out)
+    B_.hr_mask_resample(torch.as_tensor(m, device="cuda"), mout)
+    ref = img.astype(np.float64).reshape(2, 2, f, Wo, f, 3).mean((2, 4))
+    assert np.abs(out.cpu().numpy() - ref).max() <= 2e-6
+    assert (mout.cpu().numpy() == m.reshape(2, 2, f, Wo, f).max((2, 4))).all()
