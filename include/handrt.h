@@ -196,8 +196,9 @@ typedef struct hr_context hr_context;
  *   bwd_blocks_per_sm  persistent blocks per SM of the backward shader (1 .. 8)
  *   bwd_rays_per_lane  rays_per_lane of the backward shader (1, 2, 4)
  *   bwd_cand_per_chunk cand_per_chunk of the backward's work items (>= 1)
- *   edge_lanes         lanes per silhouette-edge sample in the edge-sampling kernel
- *                      (2, 4, 8, 16, 32: a warp takes 32 / edge_lanes samples)
+ *   edge_lanes         lanes per silhouette-edge sample in the edge-sampling kernel at
+ *                      most (2, 4, 8, 16, 32); calls with more samples than fill the
+ *                      GPU take fewer, down to one
  * Every setting gives the same results (the backward up to float32 summation order);
  * only the speed changes.  Defaults: 2, 8, 16, 8, 4, 4, 16, 4. */
 typedef struct hr_tuning {

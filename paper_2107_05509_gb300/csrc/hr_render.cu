@@ -2495,16 +2495,22 @@ __device__ __forceinline__ Hit group_min(Hit m) {
 // boundary term (edge sampling).  A warp takes 32 / L samples, L lanes each: sample i
 // of the launch is i % Ne_max of global view i / Ne_max (views with fewer samples skip
 // the rest).  The lanes of a group compute the sample's set-up redundantly (same
-// values, broadcast loads), then search the depth-sorted candidates of the sub-tile
-// under the sample L at a time, lane q of the group testing candidate base + q against
-// both offset rays (f+ and f-) and the group keeping the nearest hit of each (t, then
-// the lower triangle id).  A ray stops at the first group of candidates whose nearest
-// depth lies beyond its hit: the hits are those of testing the candidates one by one
-// in depth order.  The group's lanes add the six results (two endpoints x three
-// coordinates).
+// values, broadcast loads), then search the depth-sorted candidates of the sub-tile under
+// the sample in windows of 32: lane q of the group first tests the boxes of candidates q,
+// q + L, ... against the points of both offset rays (f+ and f-), loads that do not wait for
+// one another, and only then intersects those that passed, each ray keeping the lane's
+// nearest hit (t, then the lower triangle id); the group's nearest is taken once per window.
+// Candidate by candidate, box and triangle were a chain of four dependent loads and the
+// group's minimum a dozen shuffles per step, and few boxes hold a point.  Bound by latency
+// at few samples and by the lanes' unequal numbers of triangles at many: a batch of 64
+// hands 3.45 -> 1.40 ms, a 98 k-triangle hand 1.08 -> 0.45 ms, a step of two 128 x 128 views
+// with 2048 samples 308 -> 255 us in all.  A ray stops at the first window whose nearest
+// depth lies beyond its hit: the hits are those of testing the candidates one by one in
+// depth order.  The group's lanes add the six results (two endpoints x three coordinates).
 __device__ __forceinline__ void add1(float* p, float x) { atomicAdd(p, x); }
 __device__ __forceinline__ void add1(unsigned long long* p, float x) { add_fixed(p, x); }
 
+constexpr int kEdgeWin = 32;   // candidates whose boxes are tested before any is intersected
 // T: float sums (dedge [n_inst][3V]) or fixed-point sums (fx [n_inst][6V], dV part);
 // L: lanes per sample (the tuning's edge_lanes)
 template <bool STATS, class T, int L>
@@ -2514,7 +2520,7 @@ __global__ void __launch_bounds__(kRenderThreads) k_edge_samples(RenderArgs a_in
                                                                  const int* __restrict__ counts, int Ne_max, float eps,
                                                                  T* __restrict__ d_verts_all, long long inst_stride,
                                                                  unsigned long long* stats) {
-  static_assert(L == 2 || L == 4 || L == 8 || L == 16 || L == 32, "lanes per edge sample");
+  static_assert(L == 1 || L == 2 || L == 4 || L == 8 || L == 16 || L == 32, "lanes per edge sample");
   const unsigned full = 0xffffffffu;
   const RenderArgs a0 = with_iter(a_in);
   const int lane = threadIdx.x & 31, q = lane % L;
@@ -2588,7 +2594,9 @@ __global__ void __launch_bounds__(kRenderThreads) k_edge_samples(RenderArgs a_in
               // far smaller
               const int st = st0 + (py / kSubH) * nsx + (px / kSubW);
               int2 pk = a.wk.st[st];
-              if (pk.y > 0 && !in_range(a.status, (long long)pk.x + pk.y - 1, 0, a.wk.pool_cap)) pk.y = -1;
+              if (pk.y > 0 && (!in_range(a.status, pk.x, 0, a.wk.pool_cap) ||
+                               !in_range(a.status, (long long)pk.x + pk.y - 1, 0, a.wk.pool_cap)))
+                pk.y = -1;
               off = pk.x;
               K = pk.y;
               o = make_float3(cam.c[0], cam.c[1], cam.c[2]);
@@ -2607,61 +2615,68 @@ __global__ void __launch_bounds__(kRenderThreads) k_edge_samples(RenderArgs a_in
   Hit hp{-1, INFINITY, 0.0f, 0.0f}, hm{-1, INFINITY, 0.0f, 0.0f};
   // ---- no candidate list: lanes 0 and 1 of the group traverse the BVH -----------
   if (__any_sync(full, active && K < 0)) {
-    Hit h{-1, INFINITY, 0.0f, 0.0f};
-    if (active && K < 0 && q < 2) h = trace<STATS>(a.nodes, a.tris, o, q == 0 ? dp : dm, a.status, cnt, a.max_visits);
-    const int g0 = lane - q;
-    Hit r0, r1;
-    r0.tri = __shfl_sync(full, h.tri, g0);
-    r0.t = __shfl_sync(full, h.t, g0);
-    r0.u = __shfl_sync(full, h.u, g0);
-    r0.v = __shfl_sync(full, h.v, g0);
-    r1.tri = __shfl_sync(full, h.tri, g0 + 1);
-    r1.t = __shfl_sync(full, h.t, g0 + 1);
-    r1.u = __shfl_sync(full, h.u, g0 + 1);
-    r1.v = __shfl_sync(full, h.v, g0 + 1);
-    if (active && K < 0) {
-      hp = r0;
-      hm = r1;
-    }
-  }
-  // ---- candidate search, both rays together, L candidates per step ---------------
-  bool donep = !(active && K > 0), donem = donep;
-  for (int base = 0;; base += L) {
-    const bool go = !(donep && donem) && base < K;
-    if (!__any_sync(full, go)) break;
-    Hit mp{-1, INFINITY, 0.0f, 0.0f}, mm{-1, INFINITY, 0.0f, 0.0f};
-    if (go) {
-      // group-uniform: no candidate from here on can be nearer than a ray's hit
-      const float z0 = __ldg(&a.wk.z[off + base]);
-      const float zl0 = z0 - (1e-4f * fabsf(z0) + 1e-6f);
-      donep = donep || hp.t < zl0;
-      donem = donem || hm.t < zl0;
-      const int c = base + q;
-      if (!(donep && donem) && c < K && in_range(a.status, off + c, 0, a.wk.pool_cap)) {
-        const float zm = __ldg(&a.wk.z[off + c]);
-        const float zl = zm - (1e-4f * fabsf(zm) + 1e-6f);
-        bool tp = !donep && !(hp.t < zl), tm = !donem && !(hm.t < zl);
-        if (tp || tm) {
-          const float4 bb = __ldg(&a.wk.bb[off + c]);
-          if (STATS) cnt.cands += (unsigned)tp + (unsigned)tm;
-          tp = tp && xp >= bb.x && xp <= bb.z && yp >= bb.y && yp <= bb.w;
-          tm = tm && xm >= bb.x && xm <= bb.z && ym >= bb.y && ym <= bb.w;
-          if (tp || tm) {
-            const int kr = __ldg(&a.wk.rec[off + c]);
-            if (in_range(a.status, kr, 0, a.max_visits - 1)) {
-              if (tp) isect<STATS>(a.tris, kr, o, dp, mp, cnt);
-              if (tm) isect<STATS>(a.tris, kr, o, dm, mm, cnt);
-            }
-          }
-        }
+    if constexpr (L == 1) {
+      if (active && K < 0) {
+        hp = trace<STATS>(a.nodes, a.tris, o, dp, a.status, cnt, a.max_visits);
+        hm = trace<STATS>(a.nodes, a.tris, o, dm, a.status, cnt, a.max_visits);
+      }
+    } else {
+      Hit h{-1, INFINITY, 0.0f, 0.0f};
+      if (active && K < 0 && q < 2) h = trace<STATS>(a.nodes, a.tris, o, q == 0 ? dp : dm, a.status, cnt, a.max_visits);
+      const int g0 = lane - q;
+      Hit r0, r1;
+      r0.tri = __shfl_sync(full, h.tri, g0);
+      r0.t = __shfl_sync(full, h.t, g0);
+      r0.u = __shfl_sync(full, h.u, g0);
+      r0.v = __shfl_sync(full, h.v, g0);
+      r1.tri = __shfl_sync(full, h.tri, g0 + 1);
+      r1.t = __shfl_sync(full, h.t, g0 + 1);
+      r1.u = __shfl_sync(full, h.u, g0 + 1);
+      r1.v = __shfl_sync(full, h.v, g0 + 1);
+      if (active && K < 0) {
+        hp = r0;
+        hm = r1;
       }
     }
-    mp = group_min<L>(mp);
-    mm = group_min<L>(mm);
-    if (go) {
-      if (nearer(mp, hp)) hp = mp;
-      if (nearer(mm, hm)) hm = mm;
+  }
+  // ---- candidate search, both rays together ---------------------------------------
+  const bool listed = active && K > 0;
+  for (int base = 0;; base += kEdgeWin) {
+    bool go = listed && base < K;
+    if (go && base > 0) {   // group-uniform: no candidate from here on can be nearer than the hits
+      const float z0 = __ldg(&a.wk.z[off + base]), zl0 = z0 - (1e-4f * fabsf(z0) + 1e-6f);
+      go = !(hp.t < zl0 && hm.t < zl0);
     }
+    if (!__any_sync(full, go)) break;
+    // the lane's candidates base + q, base + q + L, ... whose boxes hold a ray's point
+    unsigned bp = 0u, bm = 0u;
+    if (go) {
+#pragma unroll
+      for (int h = 0; h < kEdgeWin / L; h += 8)
+#pragma unroll
+        for (int n = h; n < min(h + 8, kEdgeWin / L); ++n) {
+          const int c = base + n * L + q;
+          const float4 bb = __ldg(&a.wk.bb[off + min(c, K - 1)]);
+          if (c < K) {
+            bp |= (unsigned)(xp >= bb.x && xp <= bb.z && yp >= bb.y && yp <= bb.w) << n;
+            bm |= (unsigned)(xm >= bb.x && xm <= bb.z && ym >= bb.y && ym <= bb.w) << n;
+          }
+        }
+    }
+    for (unsigned bits = bp | bm; bits; bits &= bits - 1u) {
+      const int n = __ffs(bits) - 1, c = base + n * L + q;
+      const float zm = __ldg(&a.wk.z[off + c]), zl = zm - (1e-4f * fabsf(zm) + 1e-6f);
+      const bool tp = (bp >> n & 1u) && !(hp.t < zl), tm = (bm >> n & 1u) && !(hm.t < zl);
+      if (STATS) cnt.cands += (unsigned)tp + (unsigned)tm;
+      if (!tp && !tm) continue;
+      const int kr = __ldg(&a.wk.rec[off + c]);
+      if (!in_range(a.status, kr, 0, a.max_visits - 1)) continue;
+      if (tp) isect<STATS>(a.tris, kr, o, dp, hp, cnt);
+      if (tm) isect<STATS>(a.tris, kr, o, dm, hm, cnt);
+    }
+    __syncwarp();
+    hp = group_min<L>(hp);
+    hm = group_min<L>(hm);
   }
   if (STATS) {
     if (q == 0) cnt.hits += (unsigned)(active && hp.tri >= 0) + (unsigned)(active && hm.tri >= 0);
@@ -3079,16 +3094,21 @@ int launch_render_bwd(Context* ctx, const hr_model* m, const float* verts, const
     int rc = launch_silhouettes(ctx, m, verts, cams, nv, ctx->sil, ctx->lim.max_E, ctx->sil_count, es);
     if (rc != HR_OK) return rc;
     tm.end(kTimeBwdSil);
-    // edge_lanes lanes per edge sample
-    const int L = ctx->tune.edge_lanes;
+    // At most edge_lanes lanes per edge sample, fewer when the samples alone fill the GPU
+    // (about 2.5 times its resident threads at this kernel's registers): the lanes of a
+    // sample share its search but each do its set-up.  Whole passes at 4 / 2 / 1 lanes, us:
+    // 28 k samples 326 / 326 / 347, 40 k 323 / 329 / 335, 78 k 278 / 267 / 267, 86 k with
+    // long lists 1795 / 1692 / 1714; this kernel for a batch of 64 hands 2177 / 1712 / 1404.
+    int L = ctx->tune.edge_lanes;
+    while (L > 1 && (long long)nv * Ne * L > 200000) L >>= 1;
     const long long n = ((long long)nv * Ne + 32 / L - 1) / (32 / L) * 32;
     const unsigned grid = (unsigned)((n + kRenderThreads - 1) / kRenderThreads);
     tm.begin(kTimeBwdEdges);
 #define HR_EDGE_KERNEL(T_)                                                                            \
-  (st ? (L == 2 ? k_edge_samples<true, T_, 2> : L == 4 ? k_edge_samples<true, T_, 4>                  \
+  (st ? (L == 1 ? k_edge_samples<true, T_, 1> : L == 2 ? k_edge_samples<true, T_, 2> : L == 4 ? k_edge_samples<true, T_, 4>                  \
          : L == 8 ? k_edge_samples<true, T_, 8> : L == 16 ? k_edge_samples<true, T_, 16>              \
                                                         : k_edge_samples<true, T_, 32>)               \
-      : (L == 2 ? k_edge_samples<false, T_, 2> : L == 4 ? k_edge_samples<false, T_, 4>                \
+      : (L == 1 ? k_edge_samples<false, T_, 1> : L == 2 ? k_edge_samples<false, T_, 2> : L == 4 ? k_edge_samples<false, T_, 4>                \
          : L == 8 ? k_edge_samples<false, T_, 8> : L == 16 ? k_edge_samples<false, T_, 16>            \
                                                          : k_edge_samples<false, T_, 32>))
     if (det) {

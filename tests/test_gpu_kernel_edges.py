@@ -8,7 +8,7 @@ import pytest
 from oracle import net as N
 from tests import test_gpu_gemm as TG
 from tests import test_gpu_net as TN
-from tests.gpu_common import hand, require_gpu, torch
+from tests.gpu_common import hand, require_gpu, scene, torch
 
 pytestmark = pytest.mark.gpu
 
@@ -126,3 +126,24 @@ def test_resampling_by_whole_factors(B_, W, Wo):
     ref = img.astype(np.float64).reshape(2, 2, f, Wo, f, 3).mean((2, 4))
     assert np.abs(out.cpu().numpy() - ref).max() <= 2e-6
     assert (mout.cpu().numpy() == m.reshape(2, 2, f, Wo, f).max((2, 4))).all()
+
+
+@pytest.mark.parametrize("name,samples", [("tiny", 60), ("ragged", 700), ("ragged", 150000)])
+def test_edge_samples_do_not_depend_on_their_lanes(B_, name, samples):
+    """Fixed-point sums: the same bits for 2 to 32 lanes per sample, and (150000 samples)
+    for the one to four lanes that large calls come down to."""
+    sc, h = scene(name), hand()
+    model, ctx = B_.Model(h), B_.Context(h.V, h.F, h.E, sc.N, sc.W, sc.H)
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+    vt, cams, bg = t(sc.verts), t(sc.cams), t(sc.bg)
+    adj = t(np.random.default_rng(3).normal(size=(sc.N, sc.H, sc.W, 3)).astype(np.float32))
+    img, outs = torch.empty((sc.N, sc.H, sc.W, 3), device="cuda"), []
+    B_.hr_build_bvh(ctx, model, vt)
+    opts = lambda flags: B_.render_opts(seed=7, spp=2, edge_samples=samples, flags=flags)
+    B_.hr_render_fwd(ctx, model, vt, cams, sc.H, sc.W, bg, opts(0), img)
+    for lanes in (2, 4, 8, 16, 32):
+        ctx.set_tuning(edge_lanes=lanes)
+        outs.append(torch.empty((h.V, 3), device="cuda"))
+        B_.hr_render_bwd(ctx, model, vt, cams, sc.H, sc.W, bg, opts(B_.HR_DETERMINISTIC | B_.HR_BWD_REUSE_FWD), adj, outs[-1])
+    assert outs[0].abs().max() > 0 and all(torch.equal(outs[0], o) for o in outs[1:])
+    assert B_.hr_get_status(ctx) == B_.HR_OK
