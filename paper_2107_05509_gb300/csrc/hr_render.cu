@@ -1524,21 +1524,42 @@ __global__ void __launch_bounds__(kBinThreads) k_bin(RenderArgs a0, unsigned* __
   }
 }
 
-// Work items of the sub-tiles held by lanes 0 .. kGroupSubtiles - 1 (all lanes call): each
+// Work items of the sub-tiles held by lanes 0 .. G - 1 (all lanes call): each
 // `need` lane's sub-tile st (instance inst, candidate count K) gets C consecutive
 // items.  One reservation per instance among the lanes -- heavy items from the front
 // of the instance's region, the others from its back -- so the instance's counters
 // see one atomic per warp, not one per sub-tile.  Sub-tiles without a candidate list
 // (K < 0) are listed for k_overflow's per-ray traversal; when the region has no room
 // for a group, its sub-tiles go to k_overflow whole.
+template <int G>
 __device__ __forceinline__ void place_items(const RenderArgs& a0, bool need, int st, int inst, int K, int C,
                                             bool heavy) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int key = need ? inst : -1;
   int hx = 0, lx = 0, ht = 0, lt = 0, leader = -1;
+  const unsigned needs = __ballot_sync(full, need);
+  const int first_key = __shfl_sync(full, key, needs ? __ffs(needs) - 1 : 0);
+  if (G == 32 && __all_sync(full, !need || key == first_key)) {
+    // one instance, as a rule: sums over the lanes, both kinds in one word (C <= 16)
+    const int mine = need ? C << (heavy ? 0 : 16) : 0;
+    int incl = mine;
 #pragma unroll
-  for (int j = 0; j < kGroupSubtiles; ++j) {
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(full, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const int tot = __shfl_sync(full, incl, 31), excl = incl - mine;
+    if (need) {
+      hx = excl & 0xffff;
+      lx = excl >> 16;
+      ht = tot & 0xffff;
+      lt = tot >> 16;
+      leader = __ffs(needs) - 1;
+    }
+  } else
+#pragma unroll 8
+  for (int j = 0; j < G; ++j) {
     const int kj = __shfl_sync(full, key, j), cj = __shfl_sync(full, C, j);
     const bool hj = __shfl_sync(full, (int)heavy, j) != 0;
     if (need && kj == key) {
@@ -1581,24 +1602,27 @@ __device__ __forceinline__ void place_items(const RenderArgs& a0, bool need, int
   }
 }
 
-// Each warp takes kGroupSubtiles consecutive sub-tiles, one per lane of its first lanes.
+// Each warp takes G consecutive sub-tiles, one per lane of its first lanes: 8 to spread a
+// small call over the SMs, all 32 lanes when there is work for every warp (2.1 M sub-tiles
+// of 128 pairs 178 -> 99 us, a batch of 64 hands 222 -> 144 us).
 // A sub-tile with no record in its bin sees only the background (k_background writes
 // it).  The others get a pool range for their K records (one atomic per warp), the
 // work items of their chunks, and an entry in the list k_bin_sort orders; the count
 // becomes the fill's slot counter.  A sub-tile with more records than a list holds,
 // or whose records find no pool room, is traced ray by ray (K = -1, -(K + 1)).
+template <int G>
 __global__ void __launch_bounds__(kGroupThreads) k_bin_alloc(RenderArgs a0, unsigned* __restrict__ bin) {
   pdl_wait();
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int total = visit_count(a0);
   const int nw = gridDim.x * (kGroupThreads / 32);
-  for (int g0 = (blockIdx.x * (kGroupThreads / 32) + (threadIdx.x >> 5)) * kGroupSubtiles; g0 < total;
-       g0 += nw * kGroupSubtiles) {
+  for (int g0 = (blockIdx.x * (kGroupThreads / 32) + (threadIdx.x >> 5)) * G; g0 < total;
+       g0 += nw * G) {
     int st = -1, K = 0;
     bool listed = false;
     SubTile t{};
-    if (lane < kGroupSubtiles && g0 + lane < total) {
+    if (lane < G && g0 + lane < total) {
       const int s = visit_subtile(a0, g0 + lane);
       if (in_range(a0.status, s, 0, a0.total_st)) {
         t = subtile(a0, s);
@@ -1619,12 +1643,12 @@ __global__ void __launch_bounds__(kGroupThreads) k_bin_alloc(RenderArgs a0, unsi
     const int want = listed && K <= kLeafCap ? K : 0;
     int incl = want;
 #pragma unroll
-    for (int o = 1; o < kGroupSubtiles; o <<= 1) {
+    for (int o = 1; o < G; o <<= 1) {
       const int y = __shfl_up_sync(full, incl, o);
       if (lane >= o) incl += y;
     }
     unsigned base = 0u;
-    const int tot = __shfl_sync(full, incl, kGroupSubtiles - 1);
+    const int tot = __shfl_sync(full, incl, G - 1);
     if (lane == 0 && tot > 0) base = atomicAdd(&a0.wk.ctr[1], (unsigned)tot);
     base = __shfl_sync(full, base, 0);
     bool sorted = false, heavy = false;
@@ -1641,7 +1665,7 @@ __global__ void __launch_bounds__(kGroupThreads) k_bin_alloc(RenderArgs a0, unsi
       C = chunks_for(a0, Kc, t.spp);
       heavy = heavy_item(a0, Kc, C, t.spp);
     }
-    place_items(a0, listed, st, t.inst, Kc, C, heavy);
+    place_items<G>(a0, listed, st, t.inst, Kc, C, heavy);
     const unsigned sm = __ballot_sync(full, sorted);
     int lb = 0;
     if (lane == 0 && sm) lb = (int)atomicAdd(&a0.wk.ctr[ctr_sort(a0.n_inst)], (unsigned)__popc(sm));
@@ -1704,8 +1728,68 @@ __global__ void __launch_bounds__(kGroupThreads) k_background(RenderArgs a0, flo
   flush_counts<STATS>(cnt, stats);
 }
 
+// A list of K <= 32 E records sorted by (depth, place in the list), E per lane in
+// registers: the keys by a bitonic network (strides below E within a lane, the others by
+// shuffles), then every record fetched from its place before any is written.  In shared
+// memory each of the 21 (or 28) stages cost two dependent accesses and a barrier, and the
+// boxes were projected again: 128 pairs of views 560 -> 319 us, 64 hands 452 -> 275 us (with
+// lists up to 32, which one register per lane holds, unchanged).
+template <int E>
+__device__ __forceinline__ void sort_in_registers(const RenderArgs& a, int off, int K) {
+  typedef unsigned long long u64;
+  const int lane = threadIdx.x & 31;
+  u64 r[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = lane + 32 * e;
+    r[e] = ~0ull;
+    if (i < K) {   // unsigned order of the bits = the floats' order
+      const unsigned b = __float_as_uint(a.wk.z[off + i]);
+      r[e] = (u64)(b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u)) << 32 | (unsigned)i;
+    }
+  }
+#pragma unroll
+  for (int size = 2; size <= 32 * E; size <<= 1)
+#pragma unroll
+    for (int j = size >> 1; j > 0; j >>= 1)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {   // lane's keys E lane .. E lane + E - 1
+        const bool up = size < E ? !(e & size) : !((lane * E) & size);
+        if (j >= E) {
+          const u64 o = __shfl_xor_sync(0xffffffffu, r[e], j / E);
+          const bool low = (!((lane * E) & j)) == up;
+          if ((o < r[e]) == low) r[e] = o;
+        } else if (!(e & j)) {
+          const u64 lo = min(r[e], r[e + j]), hi = max(r[e], r[e + j]);
+          r[e] = up ? lo : hi;
+          r[e + j] = up ? hi : lo;
+        }
+      }
+  int k[E];
+  unsigned pm[E];
+  float4 bb[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = off + (lane * E + e < K ? (int)(unsigned)r[e] : 0);
+    k[e] = a.wk.rec[i];
+    pm[e] = a.wk.pm[i];
+    bb[e] = a.wk.bb[i];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = lane * E + e;
+    if (i >= K) continue;
+    const unsigned b = (unsigned)(r[e] >> 32);
+    a.wk.bb[off + i] = bb[e];
+    a.wk.z[off + i] = __uint_as_float(b ^ ((b >> 31) ? 0x80000000u : 0xffffffffu));
+    a.wk.rec[off + i] = k[e];
+    a.wk.pm[off + i] = pm[e];
+  }
+}
+
 // one warp per listed sub-tile: its K records (in fill order) sorted by nearest depth
-// (bitonic, padded with +inf: across the lanes' registers for K <= 32, else in shared
+// (bitonic, padded with +inf: across the lanes' registers for K <= 128, else in shared
 // memory, the boxes then projected again from the records), written back in order
 struct SortSmem {   // per warp
   int leaf[kLeafCap];
@@ -1765,6 +1849,14 @@ __global__ void __launch_bounds__(kRenderThreads) k_bin_sort(RenderArgs a0) {
         a0.wk.rec[off + lane] = kc;
         a0.wk.pm[off + lane] = pc;
       }
+      continue;
+    }
+    if (K <= 64) {
+      sort_in_registers<2>(a0, off, K);
+      continue;
+    }
+    if (K <= 128) {
+      sort_in_registers<4>(a0, off, K);
       continue;
     }
     const SubTile t = subtile(a0, st);
@@ -2002,7 +2094,7 @@ __global__ void __launch_bounds__(kGroupThreads, 4) k_items_bwd(RenderArgs a0, c
     const bool need = ok && ((live >> lane) & 1u) && pk.y != 0;
     const int C = need ? chunks_for(a0, pk.y, t.spp) : 0;
     const bool heavy = need && heavy_item(a0, pk.y, C, t.spp);
-    place_items(a0, need, st, t.inst, pk.y, C, heavy);
+    place_items<kGroupSubtiles>(a0, need, st, t.inst, pk.y, C, heavy);
   }
   write_face_records(a0);   // for the shader that follows
   flush_counts<STATS>(cnt, stats);
@@ -2911,7 +3003,9 @@ int launch_render_fwd(Context* ctx, const hr_model* m, const float* verts, const
     launch_pdl(k_bin<false>, dim3(std::max(bin_blocks, 1)), dim3(kBinThreads), 0, s, a, ctx->bin_cnt);
     HR_CHECK_LAUNCH();
     const int group_blocks = ctx->num_sms * 8;
-    launch_pdl(k_bin_alloc, dim3(group_blocks), dim3(kGroupThreads), 0, s, a, ctx->bin_cnt);
+    // full warps from 16 of them per SM on (a 98 k-triangle hand at 16 x 1024^2, 524 k sub-tiles: 45 -> 30 us)
+    launch_pdl(a.total_st >= 32 * 16 * ctx->num_sms ? k_bin_alloc<32> : k_bin_alloc<8>, dim3(group_blocks), dim3(kGroupThreads),
+               0, s, a, ctx->bin_cnt);
     HR_CHECK_LAUNCH();
     if (fork && (cudaEventRecord(ctx->ev_fork, s) != cudaSuccess || cudaStreamWaitEvent(bs, ctx->ev_fork, 0) != cudaSuccess))
       return HR_ERR_CUDA;

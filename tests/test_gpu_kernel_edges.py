@@ -147,3 +147,28 @@ def test_edge_samples_do_not_depend_on_their_lanes(B_, name, samples):
         B_.hr_render_bwd(ctx, model, vt, cams, sc.H, sc.W, bg, opts(B_.HR_DETERMINISTIC | B_.HR_BWD_REUSE_FWD), adj, outs[-1])
     assert outs[0].abs().max() > 0 and all(torch.equal(outs[0], o) for o in outs[1:])
     assert B_.hr_get_status(ctx) == B_.HR_OK
+
+
+@pytest.mark.parametrize("width", [208, 104, 56, 24])
+def test_lists_of_every_length(B_, width):
+    """Sub-tiles of a hand seen ever smaller: lists of up to 32, 64, 128 and more records
+    (sorted in one, two or four registers per lane, or in shared memory) and beyond what a
+    list holds.  Pixels against the oracle's, with its tolerance."""
+    import oracle
+    from tests.gpu_common import pixel_ok
+    sc, h = scene("tiny"), hand()
+    model = B_.Model(h)
+    f = width / sc.W
+    cams = np.array(sc.cams, np.float32, copy=True)
+    cams[:, :4] *= f    # fx, fy, cx, cy
+    H = int(sc.H * f)
+    ctx = B_.Context(h.V, h.F, h.E, sc.N, width, H)
+    bg = np.random.default_rng(width).random((sc.N, H, width, 3), dtype=np.float32)
+    o = sc.opts()
+    ref = oracle.render_fwd(sc.verts, h.faces, sc.normals, h.albedo, cams, H, width, bg, o)
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+    img = torch.empty((sc.N, H, width, 3), device="cuda")
+    B_.hr_build_bvh(ctx, model, t(sc.verts))
+    B_.hr_render_fwd(ctx, model, t(sc.verts), t(cams), H, width, t(bg), sc.gpu_opts(o), img)
+    assert pixel_ok(img.cpu().numpy(), ref).all()
+    assert B_.hr_get_status(ctx) == B_.HR_OK
