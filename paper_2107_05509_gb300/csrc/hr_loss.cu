@@ -419,18 +419,30 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_ct(const float* __restric
 }
 
 // loss = scale sum_views sum_blocks |d| (double, fixed order); dT[view] = its partials
-__global__ void k_loss_ct_final(const float* __restrict__ part, int N, int nb, const float* __restrict__ scale_p,
-                                float* __restrict__ loss, float* __restrict__ dT) {
-  if (threadIdx.x < 9 * N && dT) {
-    const int view = threadIdx.x / 9, k = threadIdx.x % 9;
+// blocks 0 .. N - 1: a view's dT, warp k its k-th entry; block N: the loss, every partial in
+// double.  One thread that added the loss's 512 partials one after the other took 37 us.
+constexpr int kCtFinalThreads = 9 * 32;
+__global__ void __launch_bounds__(kCtFinalThreads) k_loss_ct_final(const float* __restrict__ part, int N, int nb,
+                                                                   const float* __restrict__ scale_p, float* __restrict__ loss,
+                                                                   float* __restrict__ dT) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (blockIdx.x < (unsigned)N) {
+    if (!dT) return;
+    const int view = blockIdx.x;
     float x = 0.0f;
-    for (int b = 0; b < nb; ++b) x += part[((size_t)view * nb + b) * kCtVals + 1 + k];
-    dT[view * 9 + k] = x;
+    for (int b = lane; b < nb; b += 32) x += part[((size_t)view * nb + b) * kCtVals + 1 + warp];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) dT[view * 9 + warp] = x;
+    return;
   }
+  __shared__ double red[kCtFinalThreads / 32];
+  double tot = 0.0;
+  for (int i = threadIdx.x; i < N * nb; i += kCtFinalThreads) tot += part[(size_t)i * kCtVals];
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, o);
+  if (lane == 0) red[warp] = tot;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    double tot = 0.0;
-    for (int v = 0; v < N; ++v)
-      for (int b = 0; b < nb; ++b) tot += part[((size_t)v * nb + b) * kCtVals];
+    for (int w = 1; w < kCtFinalThreads / 32; ++w) tot += red[w];
     loss[0] = (float)(tot * (double)scale_p[0]);
   }
 }
@@ -780,8 +792,7 @@ int launch_loss_ct(Context* ctx, const float* image, const float* obs, const uin
   HR_CHECK_LAUNCH();
   k_loss_ct<<<dim3(kCtBlocks, N), kLossThreads, 0, s>>>(image, obs, mask, T, HW, scale, adjoint, ctx->ct_partials);
   HR_CHECK_LAUNCH();
-  k_loss_ct_final<<<1, 32 * ((9 * N + 31) / 32 > 0 ? (9 * N + 31) / 32 : 1), 0, s>>>(ctx->ct_partials, N, kCtBlocks,
-                                                                                     scale, loss, dT);
+  k_loss_ct_final<<<N + 1, kCtFinalThreads, 0, s>>>(ctx->ct_partials, N, kCtBlocks, scale, loss, dT);
   HR_CHECK_LAUNCH();
   return HR_OK;
 }
