@@ -1730,12 +1730,13 @@ __global__ void __launch_bounds__(kGroupThreads) k_background(RenderArgs a0, flo
 
 // A list of K <= 32 E records sorted by (depth, place in the list), E per lane in
 // registers: the keys by a bitonic network (strides below E within a lane, the others by
-// shuffles), then every record fetched from its place before any is written.  In shared
-// memory each of the 21 (or 28) stages cost two dependent accesses and a barrier, and the
-// boxes were projected again: 128 pairs of views 560 -> 319 us, 64 hands 452 -> 275 us (with
-// lists up to 32, which one register per lane holds, unchanged).
+// shuffles), then the boxes and the records through the warp's shared memory to their new
+// places.  With the keys in shared memory each of the 21 to 45 stages cost two dependent
+// accesses and a barrier, and the boxes were projected again: 128 pairs of views 560 -> 235
+// us, 64 hands 452 -> 264 us, a 98 k-triangle hand 178 -> 57 us, two views of 128 x 128
+// (lists of up to 500) 68 -> 15 us.
 template <int E>
-__device__ __forceinline__ void sort_in_registers(const RenderArgs& a, int off, int K) {
+__device__ __forceinline__ void sort_in_registers(const RenderArgs& a, int off, int K, float4* sm) {
   typedef unsigned long long u64;
   const int lane = threadIdx.x & 31;
   u64 r[E];
@@ -1748,59 +1749,67 @@ __device__ __forceinline__ void sort_in_registers(const RenderArgs& a, int off, 
       r[e] = (u64)(b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u)) << 32 | (unsigned)i;
     }
   }
+  // (loops over the stages: unrolled, 16 keys are 70 KB of instructions, which a warp reads
+  // once and waits for)
+#pragma unroll 1
+  for (int size = 2; size <= 32 * E; size <<= 1) {
+#pragma unroll 1
+    for (int j = size >> 1; j >= E; j >>= 1) {
+      const bool low = !((lane * E) & j) == !((lane * E) & size);   // this lane keeps the smaller keys
 #pragma unroll
-  for (int size = 2; size <= 32 * E; size <<= 1)
+      for (int e = 0; e < E; ++e) {
+        const u64 o = __shfl_xor_sync(0xffffffffu, r[e], j / E);
+        if ((o < r[e]) == low) r[e] = o;
+      }
+    }
 #pragma unroll
-    for (int j = size >> 1; j > 0; j >>= 1)
+    for (int j = E / 2; j > 0; j >>= 1) {
+      if (j > size >> 1) continue;
 #pragma unroll
       for (int e = 0; e < E; ++e) {   // lane's keys E lane .. E lane + E - 1
-        const bool up = size < E ? !(e & size) : !((lane * E) & size);
-        if (j >= E) {
-          const u64 o = __shfl_xor_sync(0xffffffffu, r[e], j / E);
-          const bool low = (!((lane * E) & j)) == up;
-          if ((o < r[e]) == low) r[e] = o;
-        } else if (!(e & j)) {
-          const u64 lo = min(r[e], r[e + j]), hi = max(r[e], r[e + j]);
-          r[e] = up ? lo : hi;
-          r[e + j] = up ? hi : lo;
-        }
+        if (e & j) continue;
+        const bool up = !((lane * E + e) & size), swap = (r[e + j] < r[e]) == up;
+        const u64 x = r[e], y = r[e + j];
+        r[e] = swap ? y : x;
+        r[e + j] = swap ? x : y;
       }
-  int k[E];
-  unsigned pm[E];
-  float4 bb[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int i = off + (lane * E + e < K ? (int)(unsigned)r[e] : 0);
-    k[e] = a.wk.rec[i];
-    pm[e] = a.wk.pm[i];
-    bb[e] = a.wk.bb[i];
+    }
   }
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (lane + 32 * e < K) sm[lane + 32 * e] = a.wk.bb[off + lane + 32 * e];
   __syncwarp();
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int i = lane * E + e;
     if (i >= K) continue;
     const unsigned b = (unsigned)(r[e] >> 32);
-    a.wk.bb[off + i] = bb[e];
+    a.wk.bb[off + i] = sm[(unsigned)r[e]];
     a.wk.z[off + i] = __uint_as_float(b ^ ((b >> 31) ? 0x80000000u : 0xffffffffu));
-    a.wk.rec[off + i] = k[e];
-    a.wk.pm[off + i] = pm[e];
   }
+  __syncwarp();
+  uint2* sr = reinterpret_cast<uint2*>(sm);
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (lane + 32 * e < K) sr[lane + 32 * e] = make_uint2((unsigned)a.wk.rec[off + lane + 32 * e], a.wk.pm[off + lane + 32 * e]);
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = lane * E + e;
+    if (i >= K) continue;
+    const uint2 v = sr[(unsigned)r[e]];
+    a.wk.rec[off + i] = (int)v.x;
+    a.wk.pm[off + i] = v.y;
+  }
+  __syncwarp();
 }
 
 // one warp per listed sub-tile: its K records (in fill order) sorted by nearest depth
-// (bitonic, padded with +inf: across the lanes' registers for K <= 128, else in shared
-// memory, the boxes then projected again from the records), written back in order
-struct SortSmem {   // per warp
-  int leaf[kLeafCap];
-  unsigned pm[kLeafCap];
-  float key[kLeafCap];
-  int idx[kLeafCap];
-};
-__global__ void __launch_bounds__(kRenderThreads) k_bin_sort(RenderArgs a0) {
+// (bitonic, padded with +inf, across the lanes' registers), written back in order
+__global__ void __launch_bounds__(kRenderThreads, 7) k_bin_sort(RenderArgs a0) {
   pdl_wait();
-  __shared__ SortSmem ssm[kWarps];
-  SortSmem& ss = ssm[threadIdx.x >> 5];
+  __shared__ float4 staged[kWarps][kLeafCap];
+  float4* sm = staged[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const int n = (int)min(*reinterpret_cast<volatile unsigned*>(&a0.wk.ctr[ctr_sort(a0.n_inst)]),
                          (unsigned)a0.total_st);
@@ -1851,68 +1860,11 @@ __global__ void __launch_bounds__(kRenderThreads) k_bin_sort(RenderArgs a0) {
       }
       continue;
     }
-    if (K <= 64) {
-      sort_in_registers<2>(a0, off, K);
-      continue;
-    }
-    if (K <= 128) {
-      sort_in_registers<4>(a0, off, K);
-      continue;
-    }
-    const SubTile t = subtile(a0, st);
-    if (!in_range(a0.status, t.inst, 0, a0.n_inst)) continue;
-    const RenderArgs a = for_inst(a0, t.inst);
-    const Cam cam = load_cam(a.cams, t.view);
-    int P = 1;
-    while (P < K) P <<= 1;
-    for (int j = lane; j < P; j += 32) {
-      int k = 0;
-      unsigned pm = 0u;
-      float z = INFINITY;
-      if (j < K) {
-        k = a.wk.rec[off + j];
-        pm = a.wk.pm[off + j];
-        z = a.wk.z[off + j];
-        if (!in_range(a.status, k, 0, a.max_visits - 1)) k = 0;
-      }
-      ss.leaf[j] = k;
-      ss.pm[j] = pm;
-      ss.key[j] = z;
-      ss.idx[j] = j;
-    }
-    __syncwarp();
-    for (int q = 2; q <= P; q <<= 1) {
-      for (int j = q >> 1; j > 0; j >>= 1) {
-        for (int i = lane; i < P; i += 32) {
-          const int ixj = i ^ j;
-          if (ixj > i) {
-            const float zi = ss.key[i], zj = ss.key[ixj];
-            const bool up = (i & q) == 0;
-            if ((zi > zj) == up) {
-              ss.key[i] = zj;
-              ss.key[ixj] = zi;
-              const int w = ss.idx[i];
-              ss.idx[i] = ss.idx[ixj];
-              ss.idx[ixj] = w;
-            }
-          }
-        }
-        __syncwarp();
-      }
-    }
-    for (int c = lane; c < K; c += 32) {
-      int j = ss.idx[c];
-      if (!in_range(a.status, j, 0, K)) j = 0;
-      const int k = ss.leaf[j];
-      float4 bb;
-      float zm;
-      project_record(a, cam, k, bb, zm);
-      a.wk.bb[off + c] = bb;
-      a.wk.z[off + c] = zm;
-      a.wk.rec[off + c] = k;
-      a.wk.pm[off + c] = ss.pm[j];
-    }
-    __syncwarp();
+    if (K <= 64) sort_in_registers<2>(a0, off, K, sm);
+    else if (K <= 128) sort_in_registers<4>(a0, off, K, sm);
+    else if (K <= 256) sort_in_registers<8>(a0, off, K, sm);
+    else sort_in_registers<16>(a0, off, K, sm);
+    static_assert(kLeafCap <= 512, "16 records per lane");
   }
 }
 
