@@ -20,7 +20,8 @@ namespace hr {
 
 namespace {
 
-constexpr int kSkinThreads = 256;
+constexpr int kSkinThreads = 256;   // of the adjoint
+constexpr int kSkinVerts = 128;     // vertices (and threads) of a block of the forward
 
 struct Chain {
   float Rl[kMaxJ][9];   // local rotations
@@ -111,11 +112,11 @@ struct ModelArgs {
 
 // joint j's parent as the chain uses it: parents must precede children and only joint
 // 0 is a root; a parent that breaks this is taken as joint 0 (as -1 for joint 0) and
-// reported (report = true) in the status word
-__device__ __forceinline__ int chain_parent(const ModelArgs& m, int j, int* status, bool report) {
+// reported in the status word
+__device__ __forceinline__ int chain_parent(const ModelArgs& m, int j, int* status) {
   int p = m.parents[j];
   if (p >= j || p < -1 || (j == 0) != (p < 0)) {
-    if (report) set_status(status, kStatusBadModel);
+    set_status(status, kStatusBadModel);
     p = j == 0 ? -1 : 0;
   }
   return p;
@@ -131,14 +132,14 @@ __device__ void build_chain(const ModelArgs& m, const float* __restrict__ params
   if (tid < 61 && !isfinite(params[tid])) set_status(status, kStatusNonfinite);
   if (tid < m.K) ch.beta[tid] = params[tid];
   if (tid < 3) ch.tau[tid] = params[58 + tid];
-  if (tid < m.J) {   // depth of joint j (a chain of checked parents ends within j steps)
-    const int p = chain_parent(m, tid, status, true);
+  if (tid < m.J) ch.par[tid] = chain_parent(m, tid, status);
+  __syncthreads();
+  if (tid < m.J) {   // depth of joint j (a walk over the checked parents ends within j steps; over
+                     // those in memory it was a chain of their latencies)
     int d = 0;
-    for (int q = p; q >= 0; q = chain_parent(m, q, status, false)) ++d;
-    ch.par[tid] = p;
+    for (int q = ch.par[tid]; q >= 0; q = ch.par[q]) ++d;
     ch.depth[tid] = d;
   }
-  __syncthreads();
   if (tid < 3 * m.J) {
     const int j = tid / 3, c = tid % 3;
     const float* row = m.j_shapedirs + (3 * j + c) * m.K;
@@ -157,6 +158,7 @@ __device__ void build_chain(const ModelArgs& m, const float* __restrict__ params
     float rr[3] = {r[0], r[1], r[2]};
     rodrigues(rr, ch.Rl[j]);
   }
+  __syncthreads();
   if (tid == 0) {
     int d = 0;
     for (int j = 0; j < m.J; ++j) d = max(d, ch.depth[j]);
@@ -187,6 +189,29 @@ __device__ void build_chain(const ModelArgs& m, const float* __restrict__ params
   }
 }
 
+// Blendshape rows [n][3 K] and skinning weights [n][J] of vertices v0 .. v0 + n - 1 into
+// shared memory, lanes along the rows, without waiting: threads that read their own
+// vertex's 46 values touched a line per lane and load (forward of 128 hands 14 -> 11 us, of
+// one 9.5 -> 8.2; the adjoint gained nothing, its time is in the sums and the chain).
+__device__ __forceinline__ void copy4(float* dst, const float* src) {   // without waiting for it
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void stage_rows(const ModelArgs& m, int v0, int n, float* S) {
+  const float* row = m.shapedirs + (size_t)3 * v0 * m.K;
+  for (int i = threadIdx.x; i < n * 3 * m.K; i += blockDim.x) copy4(S + i, row + i);
+}
+__device__ __forceinline__ void stage_weights(const ModelArgs& m, int v0, int n, float (*w)[kMaxJ + 1]) {
+  const float* wt = m.weights + (size_t)v0 * m.J;
+  const int du = blockDim.x / m.J, dj = blockDim.x % m.J;
+  int u = threadIdx.x / m.J, j = threadIdx.x % m.J;
+  for (int i = threadIdx.x; i < n * m.J; i += blockDim.x) {
+    copy4(&w[u][j], wt + i);
+    u += du;
+    j += dj;
+    if (j >= m.J) j -= m.J, ++u;
+  }
+}
+__device__ __forceinline__ void wait_copies() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // vertex v's rows of the blendshape basis, S[c][k] = shapedirs[3v + c][k] (zero for
 // k >= K) and its skinning weights wv[j] (zero for j >= J): loaded up front so that
 // the loads are in flight together (loops over the run-time K and J issue them one
@@ -215,11 +240,24 @@ __device__ __forceinline__ float3 shaped_vertex(const ModelArgs& m, const Chain&
   }
   return make_float3(p[0], p[1], p[2]);
 }
+// likewise from a row in shared memory
+__device__ __forceinline__ float3 shaped_vertex(const ModelArgs& m, const Chain& ch, int v, const float* S) {
+  float p[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float acc = __ldg(m.v_template + 3 * v + c);
+#pragma unroll
+    for (int k = 0; k < kMaxK; ++k)
+      if (k < m.K) acc += S[c * m.K + k] * ch.beta[k];
+    p[c] = acc;
+  }
+  return make_float3(p[0], p[1], p[2]);
+}
 
 // blockIdx.y selects the instance: params [61] and verts [V][3] of instance y; block 0
 // also writes the posed joints G_J (each joint frame's origin plus the root
 // translation, [J][3]) when `joints_all` is given
-__global__ void __launch_bounds__(kSkinThreads) k_skin(ModelArgs m, const float* __restrict__ params_all,
+__global__ void __launch_bounds__(kSkinVerts) k_skin(ModelArgs m, const float* __restrict__ params_all,
                                                        float* __restrict__ verts_all, float* __restrict__ joints_all,
                                                        int* status, const int* __restrict__ active) {
   pdl_wait();
@@ -227,20 +265,27 @@ __global__ void __launch_bounds__(kSkinThreads) k_skin(ModelArgs m, const float*
   if (active && !active[blockIdx.y]) return;   // a retired instance of a batch
   const float* params = params_all + (size_t)blockIdx.y * 61;
   float* verts = verts_all + (size_t)blockIdx.y * 3 * m.V;
+  __shared__ float sS[kSkinVerts * 3 * kMaxK];
+  __shared__ float sw[kSkinVerts][kMaxJ + 1];
+  const int v0 = blockIdx.x * kSkinVerts;
+  stage_rows(m, v0, min(kSkinVerts, m.V - v0), sS);   // on their way beside the chain
+  stage_weights(m, v0, min(kSkinVerts, m.V - v0), sw);
   build_chain(m, params, ch, status);
   if (joints_all && blockIdx.x == 0 && threadIdx.x < 3 * m.J) {
     const int j = threadIdx.x / 3, c = threadIdx.x % 3;
     joints_all[((size_t)blockIdx.y * m.J + j) * 3 + c] = ch.tG[j][c] + ch.tau[c];
   }
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < m.V; v += gridDim.x * blockDim.x) {
-    float S[3][kMaxK], wv[kMaxJ];
-    load_vertex_rows(m, v, S, wv);
-    float3 p = shaped_vertex(m, ch, v, S);
+  wait_copies();
+  __syncthreads();
+  const int v = v0 + threadIdx.x;
+  if (v < m.V) {
+    float3 p = shaped_vertex(m, ch, v, sS + threadIdx.x * 3 * m.K);
     float out[3] = {ch.tau[0], ch.tau[1], ch.tau[2]};
 #pragma unroll
     for (int j = 0; j < kMaxJ; ++j) {
-      const float wj = wv[j];
-      if (j >= m.J || wj == 0.0f) continue;
+      if (j >= m.J) continue;
+      const float wj = sw[threadIdx.x][j];
+      if (wj == 0.0f) continue;
       for (int a = 0; a < 3; ++a)
         out[a] += wj * (ch.RA[j][3 * a] * p.x + ch.RA[j][3 * a + 1] * p.y + ch.RA[j][3 * a + 2] * p.z + ch.tA[j][a]);
     }
@@ -481,8 +526,8 @@ ModelArgs model_args(const hr_model* m) {
 }  // namespace
 
 int launch_skin(Context* ctx, const hr_model* m, const float* params, float* verts, float* joints, cudaStream_t s) {
-  int blocks = (m->V + kSkinThreads - 1) / kSkinThreads;
-  launch_pdl(k_skin, dim3(blocks, ctx->n_inst), dim3(kSkinThreads), 0, s, model_args(m), params, verts, joints,
+  int blocks = (m->V + kSkinVerts - 1) / kSkinVerts;
+  launch_pdl(k_skin, dim3(blocks, ctx->n_inst), dim3(kSkinVerts), 0, s, model_args(m), params, verts, joints,
              ctx->status, (const int*)ctx->active);
   HR_CHECK_LAUNCH();
   return HR_OK;

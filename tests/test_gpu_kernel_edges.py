@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 from oracle import net as N
+from paper_2107_05509_gb300 import inputs as I
 from tests import test_gpu_gemm as TG
 from tests import test_gpu_net as TN
 from tests.gpu_common import hand, require_gpu, scene, torch
@@ -172,3 +173,34 @@ def test_lists_of_every_length(B_, width):
     B_.hr_render_fwd(ctx, model, t(sc.verts), t(cams), H, width, t(bg), sc.gpu_opts(o), img)
     assert pixel_ok(img.cpu().numpy(), ref).all()
     assert B_.hr_get_status(ctx) == B_.HR_OK
+
+
+@pytest.mark.parametrize("n", [1, 3, 40])
+@pytest.mark.parametrize("V", [31, 128, 129, 778])
+def test_skinning_blocks(B_, V, n):
+    """Skinning and its adjoint for a model of V vertices at the edges of a block's (128 of
+    the forward): against the oracle per hand.  Forward: float32 sums of 26
+    terms of size ~0.1, 1e-6.  Adjoint: sums of V terms, 1e-5 of the largest."""
+    import oracle
+    h = hand()
+    faces = h.faces[(h.faces < V).all(1)] if V < h.V else h.faces
+    if len(faces) == 0:
+        faces = np.array([[0, 1, 2]], np.int32)
+    edges, ef, vfo, vff = I.mesh_topology(faces, V)
+    h = dataclasses.replace(h, v_template=h.v_template[:V], shapedirs=h.shapedirs[:V], weights=h.weights[:V],
+                            faces=np.ascontiguousarray(faces), edges=edges, edge_faces=ef, vf_offsets=vfo, vf_faces=vff,
+                            albedo=h.albedo[:V], uv=None)
+    model = B_.Model(h)
+    rng = np.random.default_rng(V + n)
+    x = np.concatenate([rng.normal(0, 1, (n, 10)), rng.normal(0, 0.4, (n, 48)), rng.normal(0, 0.1, (n, 3))], 1)
+    x = x.astype(np.float32)
+    g = rng.normal(size=(n, V, 3)).astype(np.float32)
+    bt = B_.Batch(h.V, h.F, h.E, [(1, 8, 8, 1, 0, i) for i in range(n)])
+    verts, dx = torch.empty((n, V, 3), device="cuda"), torch.empty((n, 61), device="cuda")
+    B_.hr_skin_batch(bt, model, torch.as_tensor(x, device="cuda"), verts)
+    B_.hr_skin_bwd_batch(bt, model, torch.as_tensor(x, device="cuda"), torch.as_tensor(g, device="cuda"), dx)
+    for i in range(n):
+        ref = oracle.skin(h, x[i].astype(np.float64))
+        assert np.abs(verts[i].cpu().numpy() - ref).max() <= 1e-6
+        d = oracle.skin_bwd(h, x[i].astype(np.float64), g[i].astype(np.float64))
+        assert np.abs(dx[i].cpu().numpy() - d).max() <= 1e-5 * max(np.abs(d).max(), 1.0)
