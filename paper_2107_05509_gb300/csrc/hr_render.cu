@@ -906,7 +906,10 @@ __device__ __forceinline__ unsigned tri_pixel_mask(float4 b, const ScreenTri& t,
 // s = o - v0, q = s x e1 and e2 . q only depend on the candidate; they are computed
 // once (the same operations, so the same float32 values) instead of once per ray.
 // Arrays of float4: lanes reading neighbouring candidates meet no bank conflict.
-constexpr int kCandCap = 48;
+// 32 of them, a window of a longer list (a tile of 48, with two masks per lane, took 9 % more
+// of a batch of 64 hands: 10.3 -> 9.4 ms).
+constexpr int kCandCap = 32;
+static_assert(kCandCap >= 32, "longer lists pass through the tile in windows of 32");
 struct CandTile {
   float4 e1[kCandCap];   // e1, depth below which no ray's hit lets the candidate matter
   float4 e2[kCandCap];   // e2, triangle id
@@ -914,10 +917,10 @@ struct CandTile {
   float4 q[kCandCap];    // q
 };
 
-// candidates [c0, c0 + n), n <= 32, of the list at `off` into slots slot0 .. (one per
-// lane); returns the lane's pixel's candidates, bit i = slot slot0 + i
+// candidates [c0, c0 + n), n <= 32, of the list at `off` into the tile (one per lane);
+// returns the lane's pixel's candidates, bit i = slot i
 template <bool STATS>
-__device__ __forceinline__ unsigned stage_candidates(const RenderArgs& a, CandTile& ct, int slot0, int off, int c0, int n,
+__device__ __forceinline__ unsigned stage_candidates(const RenderArgs& a, CandTile& ct, int off, int c0, int n,
                                                      float3 o, Counts& cnt) {
   const int lane = threadIdx.x & 31;
   unsigned pm = 0u;
@@ -932,10 +935,10 @@ __device__ __forceinline__ unsigned stage_candidates(const RenderArgs& a, CandTi
       const float3 e1 = make_float3(ta.w, tb.x, tb.y), e2 = make_float3(tb.z, tb.w, tc.x);
       const float3 s = dsub(o, xyz(ta)), q = dcross(s, e1);
       if (!in_range(a.status, __float_as_int(tc.y), 0, a.max_visits - 1)) pm = 0u;
-      ct.e1[slot0 + lane] = make_float4(e1.x, e1.y, e1.z, z - (1e-4f * fabsf(z) + 1e-6f));
-      ct.e2[slot0 + lane] = make_float4(e2.x, e2.y, e2.z, tc.y);
-      ct.s[slot0 + lane] = make_float4(s.x, s.y, s.z, ddot(e2, q));
-      ct.q[slot0 + lane] = make_float4(q.x, q.y, q.z, 0.0f);
+      ct.e1[lane] = make_float4(e1.x, e1.y, e1.z, z - (1e-4f * fabsf(z) + 1e-6f));
+      ct.e2[lane] = make_float4(e2.x, e2.y, e2.z, tc.y);
+      ct.s[lane] = make_float4(s.x, s.y, s.z, ddot(e2, q));
+      ct.q[lane] = make_float4(q.x, q.y, q.z, 0.0f);
     } else {
       pm = 0u;
     }
@@ -944,7 +947,7 @@ __device__ __forceinline__ unsigned stage_candidates(const RenderArgs& a, CandTi
   return warp_transpose32(pm);
 }
 
-// Walk of the candidates in m (bit i = slot slot0 + i, in depth order) by a lane's S
+// Walk of the candidates in m (bit i = slot i, in depth order) by a lane's S
 // rays: the float32 Moller-Trumbore test and closest-hit rule of mt_hit / trace, with
 // the candidate's part taken from the tile.  u, v >= 0 and u + v <= 1 imply u <= 1, and
 // det = 0 makes u infinite or not a number, which fails the test, so both of mt_hit's
@@ -952,10 +955,10 @@ __device__ __forceinline__ unsigned stage_candidates(const RenderArgs& a, CandTi
 // the first candidate nearer than none of its hits (the list is depth-sorted).  Rays
 // that take no part start with t = -1, nearer than any hit.
 template <bool STATS, int S>
-__device__ __forceinline__ void walk_candidates(const CandTile& ct, int slot0, unsigned m, const float3 (&d)[S],
+__device__ __forceinline__ void walk_candidates(const CandTile& ct, unsigned m, const float3 (&d)[S],
                                                 Hit (&h)[S], bool& done, Counts& cnt) {
   while (m) {
-    const int i = slot0 + __ffs(m) - 1;
+    const int i = __ffs(m) - 1;
     m &= m - 1u;
     const float4 c1 = ct.e1[i];
     float tmax = h[0].t;
@@ -991,40 +994,38 @@ struct WarpTile {
 };
 
 // sub-tile t and its first kCandCap candidates into the warp's tile (all lanes call);
-// m0, m1: the lane's pixel's candidates in slots 0-31 and 32-63
+// m0: the lane's pixel's candidates, bit i = slot i
 template <bool STATS>
 __device__ __forceinline__ void stage_tile(const RenderArgs& a, WarpTile& wt, const SubTile& t, int off, int K, unsigned& m0,
-                                           unsigned& m1, Counts& cnt) {
+                                           Counts& cnt) {
   __syncwarp();   // every lane is done with the sub-tile before
   if ((threadIdx.x & 31) == 0) wt.t = t;
   const Cam& cam = warp_cam(&wt.cam, a.cams, t.view);
-  m0 = m1 = 0u;
+  m0 = 0u;
   if (K <= 0 || K > kCandCap) return;
   const float3 o = make_float3(cam.c[0], cam.c[1], cam.c[2]);
-  m0 = stage_candidates<STATS>(a, wt.cand, 0, off, 0, min(K, 32), o, cnt);
-  if (K > 32) m1 = stage_candidates<STATS>(a, wt.cand, 32, off, 32, K - 32, o, cnt);
+  m0 = stage_candidates<STATS>(a, wt.cand, off, 0, K, o, cnt);
 }
 
 // closest hits of S rays of this lane's pixel among the K candidates at `off` (all
 // lanes call; `in`: the lane takes part).  Lists of up to kCandCap are in the tile
-// (m0, m1 from stage_tile); longer ones go through it in windows.
+// (m0 from stage_tile); longer ones go through it in windows.
 template <bool STATS, int S>
-__device__ __forceinline__ void closest_staged(const RenderArgs& a, WarpTile& wt, int off, int K, unsigned m0, unsigned m1,
+__device__ __forceinline__ void closest_staged(const RenderArgs& a, WarpTile& wt, int off, int K, unsigned m0,
                                                bool in, const float3 (&d)[S], Hit (&h)[S], Counts& cnt) {
 #pragma unroll
   for (int j = 0; j < S; ++j) h[j] = Hit{-1, in ? INFINITY : -1.0f, 0.0f, 0.0f};
   bool done = !in;
   if (K <= kCandCap) {
-    if (!done) walk_candidates<STATS, S>(wt.cand, 0, m0, d, h, done, cnt);
-    if (!done) walk_candidates<STATS, S>(wt.cand, 32, m1, d, h, done, cnt);
+    if (!done) walk_candidates<STATS, S>(wt.cand, m0, d, h, done, cnt);
     __syncwarp();
     return;
   }
   const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
   for (int w = 0; w < K; w += 32) {
     if (!__any_sync(0xffffffffu, !done)) break;
-    m0 = stage_candidates<STATS>(a, wt.cand, 0, off, w, min(32, K - w), o, cnt);
-    if (!done) walk_candidates<STATS, S>(wt.cand, 0, m0, d, h, done, cnt);
+    m0 = stage_candidates<STATS>(a, wt.cand, off, w, min(32, K - w), o, cnt);
+    if (!done) walk_candidates<STATS, S>(wt.cand, m0, d, h, done, cnt);
     __syncwarp();   // every lane is done with the window
   }
 }
@@ -1032,7 +1033,7 @@ __device__ __forceinline__ void closest_staged(const RenderArgs& a, WarpTile& wt
 // Radiance of samples [s0, s0 + S) of this lane's pixel, traced together (all lanes
 // call it); added to the sums in sample order.
 template <bool STATS, int S, bool TRACE = true>
-__device__ __forceinline__ void shade_samples(const RenderArgs& a, WarpTile& wt, int off, int K, unsigned m0, unsigned m1,
+__device__ __forceinline__ void shade_samples(const RenderArgs& a, WarpTile& wt, int off, int K, unsigned m0,
                                               int s0, float3& acc, int& misses, Counts& cnt) {
   const int lane = threadIdx.x & 31;
   const int px = wt.t.x0 + (lane % kSubW), py = wt.t.y0 + (lane / kSubW);
@@ -1050,7 +1051,7 @@ __device__ __forceinline__ void shade_samples(const RenderArgs& a, WarpTile& wt,
     }
   }
   if (K > 0) {
-    closest_staged<STATS, S>(a, wt, off, K, m0, m1, valid, d, h, cnt);
+    closest_staged<STATS, S>(a, wt, off, K, m0, valid, d, h, cnt);
   } else {
     const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
 #pragma unroll
@@ -1301,7 +1302,7 @@ __device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, u
 // hits of samples [s0, s0 + S) of this lane's pixel into window entries j0 .. (all lanes
 // call it; `live` lanes take part); returns the lane's entries with a hit
 template <bool STATS, int S, bool TRACE>
-__device__ __forceinline__ unsigned trace_samples(const RenderArgs& a, GradTile& gt, int off, int K, unsigned m0, unsigned m1,
+__device__ __forceinline__ unsigned trace_samples(const RenderArgs& a, GradTile& gt, int off, int K, unsigned m0,
                                                   int s0, int j0, bool live, Counts& cnt) {
   const int lane = threadIdx.x & 31;
   const WarpTile& wt = gt.w;
@@ -1319,7 +1320,7 @@ __device__ __forceinline__ unsigned trace_samples(const RenderArgs& a, GradTile&
     }
   }
   if (K > 0) {
-    closest_staged<STATS, S>(a, gt.w, off, K, m0, m1, live, d, h, cnt);
+    closest_staged<STATS, S>(a, gt.w, off, K, m0, live, d, h, cnt);
   } else {
     const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
 #pragma unroll
@@ -1342,16 +1343,16 @@ __device__ __forceinline__ unsigned trace_samples(const RenderArgs& a, GradTile&
 // lanes call it after stage_tile), traced S at a time.  The windows and the order of a
 // window's sums depend on [s0, s1) alone.
 template <bool STATS, int S, class Sum, bool TRACE = true>
-__device__ __forceinline__ void grad_samples(const RenderArgs& a, GradTile& gt, int off, int K, unsigned m0, unsigned m1,
+__device__ __forceinline__ void grad_samples(const RenderArgs& a, GradTile& gt, int off, int K, unsigned m0,
                                              int s0, int s1, bool live, float3 g, Sum sum, Counts& cnt) {
   const float3 G = make_float3(g.x * a.sh.lrgb.x, g.y * a.sh.lrgb.y, g.z * a.sh.lrgb.z);
   for (int w0 = s0; w0 < s1; w0 += kGradWin) {
     const int n = min(kGradWin, s1 - w0);
     unsigned pend = 0u;
     int j = 0;
-    for (; j + S <= n; j += S) pend |= trace_samples<STATS, S, TRACE>(a, gt, off, K, m0, m1, w0 + j, j, live, cnt);
+    for (; j + S <= n; j += S) pend |= trace_samples<STATS, S, TRACE>(a, gt, off, K, m0, w0 + j, j, live, cnt);
     if (S > 1)
-      for (; j < n; ++j) pend |= trace_samples<STATS, 1, TRACE>(a, gt, off, K, m0, m1, w0 + j, j, live, cnt);
+      for (; j < n; ++j) pend |= trace_samples<STATS, 1, TRACE>(a, gt, off, K, m0, w0 + j, j, live, cnt);
     grad_window<STATS>(a, gt, pend, w0, G, sum, cnt);
     __syncwarp();
   }
@@ -2215,7 +2216,7 @@ __global__ void __launch_bounds__(kRenderThreads, kFwdMinBlocks) k_shade_fwd(Ren
   Counts cnt;
   Cursor cur = start_items(a0);
   int at = -1, K = 0, off = 0, slot;   // the sub-tile staged
-  unsigned m0 = 0u, m1 = 0u;
+  unsigned m0 = 0u;
   while (next_item(a0, cur, slot)) {
     const int gi = inst_ibase(a0, cur.inst) + slot;
     const int4 item = a0.wk.items[gi];
@@ -2229,16 +2230,16 @@ __global__ void __launch_bounds__(kRenderThreads, kFwdMinBlocks) k_shade_fwd(Ren
       off = pk.x;
       K = pk.y;
       const RenderArgs a = for_inst(a0, cur.inst);
-      stage_tile<STATS>(a, wt, t, off, K, m0, m1, cnt);
+      stage_tile<STATS>(a, wt, t, off, K, m0, cnt);
     }
     const RenderArgs a = for_inst(a0, cur.inst);
     int s0, s1;
     item_samples(item.y, item.z, wt.t.spp, s0, s1);
     float3 acc = make_float3(0.0f, 0.0f, 0.0f);
     int misses = 0;
-    for (; s0 + S <= s1; s0 += S) shade_samples<STATS, S, false>(a, wt, off, K, m0, m1, s0, acc, misses, cnt);
+    for (; s0 + S <= s1; s0 += S) shade_samples<STATS, S, false>(a, wt, off, K, m0, s0, acc, misses, cnt);
     if (S > 1)
-      for (; s0 < s1; ++s0) shade_samples<STATS, 1, false>(a, wt, off, K, m0, m1, s0, acc, misses, cnt);
+      for (; s0 < s1; ++s0) shade_samples<STATS, 1, false>(a, wt, off, K, m0, s0, acc, misses, cnt);
     finish_item(a, wt.t, item, gi, acc, misses, image);
   }
   flush_counts<STATS>(cnt, stats);
@@ -2248,16 +2249,15 @@ struct FwdTile {
   WarpTile w;
 };
 template <bool STATS>
-__device__ __forceinline__ void overflow_grad(const RenderArgs& a, GradTile& gt, int inst, int off, int K, unsigned m0,
-                                              unsigned m1, int s0, int s1, bool live, float3 g, Counts& cnt) {
+__device__ __forceinline__ void overflow_grad(const RenderArgs& a, GradTile& gt, int inst, int off, int K, unsigned m0, int s0, int s1, bool live, float3 g, Counts& cnt) {
   if (a.wk.det)
-    grad_samples<STATS, 1>(a, gt, off, K, m0, m1, s0, s1, live, g,
+    grad_samples<STATS, 1>(a, gt, off, K, m0, s0, s1, live, g,
                            SumWide<unsigned long long>{a.wk.fx + (size_t)inst * 6 * a.V}, cnt);
   else
-    grad_samples<STATS, 1>(a, gt, off, K, m0, m1, s0, s1, live, g, SumF32{a.wk.extra + (size_t)inst * 8 * a.V}, cnt);
+    grad_samples<STATS, 1>(a, gt, off, K, m0, s0, s1, live, g, SumF32{a.wk.extra + (size_t)inst * 8 * a.V}, cnt);
 }
 template <bool STATS>   // the forward overflow kernel never takes this branch
-__device__ __forceinline__ void overflow_grad(const RenderArgs&, FwdTile&, int, int, int, unsigned, unsigned, int, int, bool,
+__device__ __forceinline__ void overflow_grad(const RenderArgs&, FwdTile&, int, int, int, unsigned, int, int, bool,
                                               float3, Counts&) {}
 
 // The rare paths, kept out of the gather and the shaders so that their registers are
@@ -2294,19 +2294,19 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
       bool live;
       const float3 g = lane_adjoint(a, t, adjoint, live);
       const int C = chunks_for(a, pk.y, t.spp);
-      unsigned m0, m1;
-      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, m1, cnt);
+      unsigned m0;
+      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, cnt);
       for (int c = 0; c < C; ++c) {
         int s0, s1;
         item_samples(c, C, t.spp, s0, s1);
-        overflow_grad<STATS>(a, gt, t.inst, pk.x, pk.y, m0, m1, s0, s1, live, g, cnt);
+        overflow_grad<STATS>(a, gt, t.inst, pk.x, pk.y, m0, s0, s1, live, g, cnt);
       }
     } else {
       // the same chunks and the same order of sums as the work items and finish_item
       // would use, so a pixel's value does not depend on which path rendered it
       const int C = chunks_for(a, pk.y, t.spp);
-      unsigned m0, m1;
-      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, m1, cnt);
+      unsigned m0;
+      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, cnt);
       float3 tot = make_float3(0.0f, 0.0f, 0.0f);
       float tmiss = 0.0f;
       for (int c = 0; c < C; ++c) {
@@ -2314,7 +2314,7 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
         item_samples(c, C, t.spp, s0, s1);
         float3 acc = make_float3(0.0f, 0.0f, 0.0f);
         int misses = 0;
-        for (; s0 < s1; ++s0) shade_samples<STATS, 1>(a, wt, pk.x, pk.y, m0, m1, s0, acc, misses, cnt);
+        for (; s0 < s1; ++s0) shade_samples<STATS, 1>(a, wt, pk.x, pk.y, m0, s0, acc, misses, cnt);
         tot.x += acc.x;
         tot.y += acc.y;
         tot.z += acc.z;
@@ -2343,15 +2343,15 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
     if (BWD) {
       bool live;
       const float3 g = lane_adjoint(a, t, adjoint, live);
-      unsigned m0, m1;
-      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, m1, cnt);
-      overflow_grad<STATS>(a, gt, t.inst, pk.x, pk.y, m0, m1, s0, s1, live, g, cnt);
+      unsigned m0;
+      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, cnt);
+      overflow_grad<STATS>(a, gt, t.inst, pk.x, pk.y, m0, s0, s1, live, g, cnt);
     } else {
       float3 acc = make_float3(0.0f, 0.0f, 0.0f);
       int misses = 0;
-      unsigned m0, m1;
-      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, m1, cnt);
-      for (; s0 < s1; ++s0) shade_samples<STATS, 1>(a, wt, pk.x, pk.y, m0, m1, s0, acc, misses, cnt);
+      unsigned m0;
+      stage_tile<STATS>(a, wt, t, pk.x, pk.y, m0, cnt);
+      for (; s0 < s1; ++s0) shade_samples<STATS, 1>(a, wt, pk.x, pk.y, m0, s0, acc, misses, cnt);
       finish_item(a, t, item, slot, acc, misses, image);
     }
   }
@@ -2388,7 +2388,7 @@ __global__ void __launch_bounds__(kRenderThreads, kBwdMinBlocks) k_shade_bwd(Ren
   Counts cnt;
   Cursor cur = start_items(a0);
   int at = -1, K = 0, off = 0, slot;   // the sub-tile staged
-  unsigned m0 = 0u, m1 = 0u;
+  unsigned m0 = 0u;
   bool live = false;
   float3 g = make_float3(0.0f, 0.0f, 0.0f);
   while (next_item(a0, cur, slot)) {
@@ -2405,19 +2405,19 @@ __global__ void __launch_bounds__(kRenderThreads, kBwdMinBlocks) k_shade_bwd(Ren
       off = pk.x;
       K = pk.y;
       g = lane_adjoint(a, t, adjoint, live);
-      stage_tile<STATS>(a, gt.w, t, off, K, m0, m1, cnt);
+      stage_tile<STATS>(a, gt.w, t, off, K, m0, cnt);
     }
     int s0, s1;
     item_samples(item.y, item.z, gt.w.t.spp, s0, s1);
     if constexpr (ACC == kAccGlobal)
-      grad_samples<STATS, S, SumWide<double>, false>(a, gt, off, K, m0, m1, s0, s1, live, g,
+      grad_samples<STATS, S, SumWide<double>, false>(a, gt, off, K, m0, s0, s1, live, g,
                                                      SumWide<double>{a0.wk.extra64 + (size_t)inst * 6 * a0.V}, cnt);
     else if constexpr (ACC == kAccFixed)
       grad_samples<STATS, S, SumWide<unsigned long long>, false>(
-          a, gt, off, K, m0, m1, s0, s1, live, g, SumWide<unsigned long long>{a0.wk.fx + (size_t)inst * 6 * a0.V}, cnt);
+          a, gt, off, K, m0, s0, s1, live, g, SumWide<unsigned long long>{a0.wk.fx + (size_t)inst * 6 * a0.V}, cnt);
     else
       grad_samples<STATS, S, SumF32, false>(
-          a, gt, off, K, m0, m1, s0, s1, live, g,
+          a, gt, off, K, m0, s0, s1, live, g,
           SumF32{ACC == kAccDirect ? a0.wk.extra + (size_t)inst * 8 * a0.V
                                    : partials + (size_t)(blockIdx.x % nparts) * 8 * a0.V},
           cnt);
