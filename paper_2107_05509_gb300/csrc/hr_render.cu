@@ -1734,7 +1734,7 @@ __global__ void __launch_bounds__(kGroupThreads) k_background(RenderArgs a0, flo
 // shuffles), then the boxes and the records through the warp's shared memory to their new
 // places.  With the keys in shared memory each of the 21 to 45 stages cost two dependent
 // accesses and a barrier, and the boxes were projected again: 128 pairs of views 560 -> 235
-// us, 64 hands 452 -> 264 us, a 98 k-triangle hand 178 -> 57 us, two views of 128 x 128
+// us, 64 hands 452 -> 264 us, a 24.6 k-triangle hand 178 -> 57 us, two views of 128 x 128
 // (lists of up to 500) 68 -> 15 us.
 template <int E>
 __device__ __forceinline__ void sort_in_registers(const RenderArgs& a, int off, int K, float4* sm) {
@@ -2547,7 +2547,7 @@ __device__ __forceinline__ Hit group_min(Hit m) {
 // Candidate by candidate, box and triangle were a chain of four dependent loads and the
 // group's minimum a dozen shuffles per step, and few boxes hold a point.  Bound by latency
 // at few samples and by the lanes' unequal numbers of triangles at many: a batch of 64
-// hands 3.45 -> 1.40 ms, a 98 k-triangle hand 1.08 -> 0.45 ms, a step of two 128 x 128 views
+// hands 3.45 -> 1.40 ms, a 24.6 k-triangle hand 1.08 -> 0.45 ms, a step of two 128 x 128 views
 // with 2048 samples 308 -> 255 us in all.  A ray stops at the first window whose nearest
 // depth lies beyond its hit: the hits are those of testing the candidates one by one in
 // depth order.  The group's lanes add the six results (two endpoints x three coordinates).
@@ -2955,7 +2955,7 @@ int launch_render_fwd(Context* ctx, const hr_model* m, const float* verts, const
     launch_pdl(k_bin<false>, dim3(std::max(bin_blocks, 1)), dim3(kBinThreads), 0, s, a, ctx->bin_cnt);
     HR_CHECK_LAUNCH();
     const int group_blocks = ctx->num_sms * 8;
-    // full warps from 16 of them per SM on (a 98 k-triangle hand at 16 x 1024^2, 524 k sub-tiles: 45 -> 30 us)
+    // full warps from 16 of them per SM on (a 24.6 k-triangle hand at 16 x 1024^2, 524 k sub-tiles: 45 -> 30 us)
     launch_pdl(a.total_st >= 32 * 16 * ctx->num_sms ? k_bin_alloc<32> : k_bin_alloc<8>, dim3(group_blocks), dim3(kGroupThreads),
                0, s, a, ctx->bin_cnt);
     HR_CHECK_LAUNCH();
