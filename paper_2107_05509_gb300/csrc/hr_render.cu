@@ -295,13 +295,22 @@ __device__ __forceinline__ float3 tex_texel(const RenderArgs& a, int i, int j) {
   return ld3(a.tex + 3 * ((size_t)j * a.tex_w + i));
 }
 
+// Value arithmetic of the shading, every rounding spelled out: a pixel has the same bits
+// whichever kernel shades it and however the code around is compiled.  The loss's
+// adjoint is the sign of image - observation, so a last bit that moves can turn a pixel's
+// gradient round (left to the compiler's contraction, one channel of 50 million turned
+// and moved a texture gradient by 2e-4 of its norm).
+// a b + c d, the first product exact
+__device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+// the orders are those that images have always had: of the upper pair of texels the product
+// with fx is exact in red and green, that with 1 - fx in blue
 __device__ __forceinline__ float3 tex_albedo(const RenderArgs& a, const TexSample& ts) {
   const float3 t00 = tex_texel(a, ts.i0, ts.j0), t10 = tex_texel(a, ts.i1, ts.j0);
   const float3 t01 = tex_texel(a, ts.i0, ts.j1), t11 = tex_texel(a, ts.i1, ts.j1);
-  const float gx = 1.0f - ts.fx, gy = 1.0f - ts.fy;
-  return make_float3(gy * (gx * t00.x + ts.fx * t10.x) + ts.fy * (gx * t01.x + ts.fx * t11.x),
-                     gy * (gx * t00.y + ts.fx * t10.y) + ts.fy * (gx * t01.y + ts.fx * t11.y),
-                     gy * (gx * t00.z + ts.fx * t10.z) + ts.fy * (gx * t01.z + ts.fx * t11.z));
+  const float fx = ts.fx, fy = ts.fy, gx = __fsub_rn(1.0f, fx), gy = __fsub_rn(1.0f, fy);
+  return make_float3(mul_add2(gy, mul_add2(fx, t10.x, gx, t00.x), fy, mul_add2(gx, t01.x, fx, t11.x)),
+                     mul_add2(gy, mul_add2(fx, t10.y, gx, t00.y), fy, mul_add2(gx, t01.y, fx, t11.y)),
+                     mul_add2(gy, mul_add2(gx, t00.z, fx, t10.z), fy, mul_add2(gx, t01.z, fx, t11.z)));
 }
 
 // Shading record of a face, kFaceRec float4 words:
@@ -351,24 +360,31 @@ __device__ __forceinline__ void write_face_records(const RenderArgs& a);
 
 __device__ __forceinline__ float3 xyz(float4 q) { return make_float3(q.x, q.y, q.z); }
 
-__device__ __forceinline__ float3 shade(const RenderArgs& a, const Hit& h) {
+// radiance of a hit: the albedo times the light's colour, and the factor k = ka + kd sigma
+// of all three channels, whose product a sum takes unrounded
+__device__ __forceinline__ float3 shade(const RenderArgs& a, const Hit& h, float& k) {
   const float4* r = a.frec + (size_t)kFaceRec * h.tri;
   const float3 n0 = xyz(__ldg(r)), n1 = xyz(__ldg(r + 1)), n2 = xyz(__ldg(r + 2));
-  float3 nm = interp_normal(h.u, h.v, n0, n1, n2);
-  float ndl = ddot(nm, a.sh.l);
+  const float3 nm = interp_normal(h.u, h.v, n0, n1, n2);
+  const float ndl = ddot(nm, a.sh.l);
   float sigma = 0.0f;
-  if (ndl > 0.0f) sigma = ndl * rsqrtf(nm.x * nm.x + nm.y * nm.y + nm.z * nm.z);
-  float w = 1.0f - h.u - h.v;
-  float k = a.sh.ka + a.sh.kd * sigma;
+  if (ndl > 0.0f) sigma = __fmul_rn(ndl, rsqrtf(__fmaf_rn(nm.z, nm.z, mul_add2(nm.x, nm.x, nm.y, nm.y))));
+  k = __fmaf_rn(a.sh.kd, sigma, a.sh.ka);
   float3 alb;
   if (a.tex) {
     alb = tex_albedo(a, tex_coords(a, __ldg(r + 7), __ldg(r + 8), h.u, h.v));
   } else {
     const float3 a0 = xyz(__ldg(r + 3)), a1 = xyz(__ldg(r + 4)), a2 = xyz(__ldg(r + 5));
-    alb = make_float3(w * a0.x + h.u * a1.x + h.v * a2.x, w * a0.y + h.u * a1.y + h.v * a2.y,
-                      w * a0.z + h.u * a1.z + h.v * a2.z);
+    const float w = __fsub_rn(__fsub_rn(1.0f, h.u), h.v);
+    alb = make_float3(__fmaf_rn(h.v, a2.x, mul_add2(w, a0.x, h.u, a1.x)), __fmaf_rn(h.v, a2.y, mul_add2(w, a0.y, h.u, a1.y)),
+                      __fmaf_rn(h.v, a2.z, mul_add2(w, a0.z, h.u, a1.z)));
   }
-  return make_float3(alb.x * a.sh.lrgb.x * k, alb.y * a.sh.lrgb.y * k, alb.z * a.sh.lrgb.z * k);
+  return make_float3(__fmul_rn(alb.x, a.sh.lrgb.x), __fmul_rn(alb.y, a.sh.lrgb.y), __fmul_rn(alb.z, a.sh.lrgb.z));
+}
+__device__ __forceinline__ float3 radiance(const RenderArgs& a, const Hit& h) {
+  float k;
+  const float3 f = shade(a, h, k);
+  return make_float3(__fmul_rn(f.x, k), __fmul_rn(f.y, k), __fmul_rn(f.z, k));
 }
 
 __device__ __forceinline__ Cam load_cam(const Cam* cams, int view) {
@@ -1067,10 +1083,11 @@ __device__ __forceinline__ void shade_samples(const RenderArgs& a, WarpTile& wt,
     if (!valid) continue;
     if (h[j].tri >= 0) {
       if (STATS) ++cnt.hits;
-      float3 f = shade(a, h[j]);
-      acc.x += f.x;
-      acc.y += f.y;
-      acc.z += f.z;
+      float k;
+      const float3 f = shade(a, h[j], k);
+      acc.x = __fmaf_rn(f.x, k, acc.x);
+      acc.y = __fmaf_rn(f.y, k, acc.y);
+      acc.z = __fmaf_rn(f.z, k, acc.z);
     } else {
       ++misses;
     }
@@ -1088,9 +1105,9 @@ __device__ __forceinline__ void write_pixel(const RenderArgs& a, const SubTile& 
   const float fm = __fdiv_rn((float)misses, (float)t.spp);
   const float inv_spp = 1.0f / (float)t.spp;
   float3 bgc = misses ? ld3(a.bg + 3 * pix) : make_float3(0.0f, 0.0f, 0.0f);
-  image[3 * pix] = acc.x * inv_spp + bgc.x * fm;
-  image[3 * pix + 1] = acc.y * inv_spp + bgc.y * fm;
-  image[3 * pix + 2] = acc.z * inv_spp + bgc.z * fm;
+  image[3 * pix] = mul_add2(acc.x, inv_spp, bgc.x, fm);
+  image[3 * pix + 1] = mul_add2(acc.y, inv_spp, bgc.y, fm);
+  image[3 * pix + 2] = mul_add2(acc.z, inv_spp, bgc.z, fm);
 }
 
 // Where a backward's vertex sums go: vertex i's dL/dv and dL/dn, added with atomics
@@ -2732,8 +2749,8 @@ __global__ void __launch_bounds__(kRenderThreads) k_edge_samples(RenderArgs a_in
     }
   }
   if (!active || q >= 6) return;
-  const float3 fp = hp.tri >= 0 ? shade(a, hp) : ld3(a.bg + 3 * (vw.pix0 + (size_t)byp * W + bxp));
-  const float3 fm = hm.tri >= 0 ? shade(a, hm) : ld3(a.bg + 3 * (vw.pix0 + (size_t)bym * W + bxm));
+  const float3 fp = hp.tri >= 0 ? radiance(a, hp) : ld3(a.bg + 3 * (vw.pix0 + (size_t)byp * W + bxp));
+  const float3 fm = hm.tri >= 0 ? radiance(a, hm) : ld3(a.bg + 3 * (vw.pix0 + (size_t)bym * W + bxm));
   const int Ne = a0.vt ? __ldg(&a0.vt[view].ne) : Ne_max;
   const float wgt = (A.x * (fp.x - fm.x) + A.y * (fp.y - fm.y) + A.z * (fp.z - fm.z)) * ((float)nsil / (float)Ne);
   if (wgt == 0.0f) return;
