@@ -93,6 +93,7 @@ int create_ctx(const hr_limits* lim, int n, size_t views, size_t subtiles, size_
   c->lim = *lim;
   c->n_inst = n;
   c->tune = hr_tuning{2, 8, 16, 8, 4, 4, 16, 4};
+  c->waits = hr::kWaits;
   if (cudaGetDevice(&c->device) != cudaSuccess) {
     delete c;
     return HR_ERR_CUDA;
@@ -595,8 +596,14 @@ int hr_gemm_bf16(hr_context* ctx, const void* A, int lda, const void* B, int ldb
                  hr_stream stream) {
   Context* c = reinterpret_cast<Context*>(ctx);
   if (!c || !A || !B || !C || ldc < N) return HR_ERR_ARG;
-  return hr::launch_gemm(A, lda, B, ldb, M, N, K, bias, relu, C, ldc, out_bf16, splits, split_buf, c->status,
-                         (cudaStream_t)stream);
+  return hr::launch_gemm(A, lda, B, ldb, M, N, K, bias, relu, C, ldc, out_bf16, splits, split_buf,
+                         hr::Guard{c->status, c->waits}, (cudaStream_t)stream);
+}
+
+// bounds of the waits of hr_gemm_bf16 in this context (tests)
+int hr_internal_context_waits(hr_context* ctx, int64_t clocks, int stop) {
+  reinterpret_cast<Context*>(ctx)->waits = hr::Waits{clocks, stop};
+  return HR_OK;
 }
 
 int hr_vertex_mse(const float* verts, const float* ref, int V, int n, float* loss, float* d_verts,

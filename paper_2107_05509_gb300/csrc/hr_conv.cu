@@ -27,7 +27,7 @@
 // ring run on from tile to tile and the accumulators are double-buffered, so that a
 // tile's epilogue runs beside the next tiles' products.  Every mbarrier wait is bounded;
 // one that runs out sets a status bit, its role stops, the others' waits run out
-// likewise, copies in flight are waited for and tensor memory is freed.
+// likewise, copies and products in flight are waited for and tensor memory is freed.
 #include <algorithm>
 
 #include "hr_tcgen05.cuh"
@@ -151,7 +151,7 @@ struct ConvArgs {
   bf16* out;              // fwd [M][C]; dgrad [NV][2 Ho][2 Ho][C]
   const bf16* mask;       // dgrad: the layer's activations (ReLU mask), out's layout
   ConvClass cls[4];
-  int* status;
+  Guard guard;
 };
 
 // What the roles need of each K-step of a tile, worked out once per block into shared
@@ -183,8 +183,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
   extern __shared__ __align__(1024) unsigned char raw[];
   unsigned char* sA = align1024(raw);
   unsigned char* sB = sA + S * kABytes;
-  __shared__ __align__(8) uint64_t full[S], empty[S], acc_full[2], acc_empty[2];
+  __shared__ __align__(8) uint64_t full[S], empty[S], acc_full[2], acc_empty[2], drained;
   __shared__ uint32_t tmem_slot;
+  __shared__ int gave_up;
+  const Waits& waits = c.guard.waits;
   __shared__ float sbias[BN];
   __shared__ int4 rows[kTileM];
   __shared__ Step steps[kMaxSteps];
@@ -220,6 +222,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
       mbar_init(smem_u32(&acc_full[b]), 1);
       mbar_init(smem_u32(&acc_empty[b]), 128);
     }
+    mbar_init(smem_u32(&drained), 1);
+    gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (!DGRAD && threadIdx.x < BN) sbias[threadIdx.x] = c.bias[threadIdx.x];
@@ -229,6 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   bool ok = true;
+  int filled = 0;   // stages whose copies warp 0 has asked for
   if (warp == 0) {
     // the weights' tiles, and the prefetches
     const bool leader = elect_one();
@@ -243,7 +248,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
       }
       for (int st = 0; st < T; ++st, r.next<S>()) {
         const int x = steps[st].tx, y = steps[st].ty;
-        if (!(ok = mbar_wait(smem_u32(&empty[r.s]), r.phase ^ 1))) break;
+        if (!(ok = mbar_wait(smem_u32(&empty[r.s]), r.phase ^ 1, waits.clocks))) break;
+        ++filled;
         const uint32_t fb = smem_u32(&full[r.s]);
         if (leader) {
           mbar_expect_tx(fb, Cfg::kBBytes);
@@ -251,26 +257,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
         }
       }
     }
-    // the products' issue waits for every copy before the block ends; when a role gave up,
-    // a bounded wait for those in flight
-    if (!ok) {
-      for (int s = 0; s < S; ++s) mbar_wait(smem_u32(&full[s]), 0);
-      if (lane == 0) set_status(c.status, kStatusTimeout);
-    }
   } else if (warp == 1) {
     constexpr uint32_t idesc = mma_idesc(kTileM, BN);
     const bool leader = elect_one();
     const uint32_t a0 = desc_lo(smem_u32(sA)), b0 = desc_lo(smem_u32(sB));
     Ring r;
-    int it = -1;
+    int it = -1, step = 0;
     for (int tile = blockIdx.x; ok && tile < c.tiles; tile += gridDim.x)
       for (int st = 0; st < T; ++st, r.next<S>()) {
         const Step e = steps[st];
         if (e.flags & 1) {
           ++it;
-          if (!(ok = mbar_wait(smem_u32(&acc_empty[it & 1]), ((it >> 1) & 1) ^ 1))) break;
+          if (!(ok = mbar_wait(smem_u32(&acc_empty[it & 1]), ((it >> 1) & 1) ^ 1, waits.clocks))) break;
         }
-        if (!(ok = mbar_wait(smem_u32(&full[r.s]), r.phase))) break;
+        if (!(ok = step++ != waits.stop && mbar_wait(smem_u32(&full[r.s]), r.phase, waits.clocks))) break;
         tc_fence_after();
         if (leader) {
           const uint32_t a = a0 + r.s * (kABytes >> 4), b = b0 + r.s * (Cfg::kBBytes >> 4);
@@ -284,7 +284,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
           if (e.flags & 2) mma_commit(smem_u32(&acc_full[it & 1]));
         }
       }
-    if (!ok && lane == 0) set_status(c.status, kStatusTimeout);
   } else if (warp >= 2 && warp < kGatherWarp) {
     const int q = warp & 3, grp = (warp - 2) >> 2;   // tensor-memory lanes 32 q .. of this warp
     int it = 0;
@@ -308,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
           for (int n = 0; n < BN; n += 16)
             if (in) load32(c.mask + o + n, *reinterpret_cast<uint32_t(*)[8]>(&y[n / 2]));
         }
-        if (!(ok = mbar_wait(smem_u32(&acc_full[b]), use & 1))) break;
+        if (!(ok = mbar_wait(smem_u32(&acc_full[b]), use & 1, waits.clocks))) break;
         tc_fence_after();
         const uint32_t t0 = tmem + b * Cfg::kAcc + ((uint32_t)(q * 32) << 16);
 #pragma unroll
@@ -343,7 +342,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
         tc_fence_before();
         mbar_arrive(smem_u32(&acc_empty[b]));
       }
-    if (!ok && lane == 0) set_status(c.status, kStatusTimeout);
   } else if (warp >= kGatherWarp && warp < kGatherWarp + gather_warps<S>()) {
     // lane's 16-byte column of a row, 8 lanes per row, rows rr, rr + 4, ... of the tile;
     // every G-th stage
@@ -375,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
         off = ((dy << c.g.ls) + dx) * C + (k & (C - 1));
       }
       const bool used = DGRAD || q < 2 * steps[st].groups;   // the others are not read
-      if (!(ok = mbar_wait(smem_u32(&empty[r.s]), r.phase ^ 1))) break;
+      if (!(ok = mbar_wait(smem_u32(&empty[r.s]), r.phase ^ 1, waits.clocks))) break;
       if (used) {
         const bf16* p = base + off;
         const int y0 = tv ? yb + dy : Hs;   // Hs: every row is outside
@@ -394,10 +392,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv(const __grid_constant__ CU
         r.phase ^= 1;
       }
     }
-    if (!ok && lane == 0) set_status(c.status, kStatusTimeout);
+  }
+  if (!ok && lane == 0) {
+    set_status(c.guard.status, kStatusTimeout);
+    gave_up = 1;
   }
   tc_fence_before();
   __syncthreads();
+  if (gave_up) {   // (otherwise the products have waited for the copies, the epilogue for the products)
+    if (warp == 0) drain_fills<S>(full, filled);
+    if (warp == 1) {
+      if (elect_one()) mma_commit(smem_u32(&drained));
+      mbar_wait(smem_u32(&drained), 0, kWaitClocks);
+    }
+    __syncthreads();
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_free<Cfg::kCols>(tmem);
@@ -416,7 +425,7 @@ struct WgradArgs {
   int K, N;               // products (rows of dW^T), outputs
   float* part;            // [splits][K][N]
   float* bias_part;       // [splits][N]
-  int* status;
+  Guard guard;
 };
 
 template <int BN>
@@ -438,6 +447,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
   unsigned char* sB = sA + S * kABytes;
   __shared__ __align__(8) uint64_t full[S], empty[S], done;
   __shared__ uint32_t tmem_slot;
+  __shared__ int gave_up;
+  const Waits& waits = c.guard.waits;
   __shared__ float sbias[BN];
   __shared__ int4 rows[kStep];
   if (GATHER && threadIdx.x < kStep) rows[threadIdx.x] = gather_row(c.g, threadIdx.x);
@@ -457,6 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
       mbar_init(smem_u32(&empty[s]), 1 + (bias ? 4 : 0));
     }
     mbar_init(smem_u32(&done), 1);
+    gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) tmem_alloc<kCols>(smem_u32(&tmem_slot));
@@ -465,11 +477,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   bool ok = true;
+  int filled = 0;   // stages whose copies warp 0 has asked for
   if (warp == 0) {
     const bool leader = elect_one();
     Ring r;
     for (int st = 0; st < steps; ++st, r.next<S>()) {
-      if (!(ok = mbar_wait(smem_u32(&empty[r.s]), r.phase ^ 1))) break;
+      if (!(ok = mbar_wait(smem_u32(&empty[r.s]), r.phase ^ 1, waits.clocks))) break;
+      ++filled;
       const uint32_t fb = smem_u32(&full[r.s]);
       const int row = (s0 + st) * kStep;
       if (!leader) continue;
@@ -484,17 +498,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
       if (!GATHER)
         for (int h = 0; h < 2; ++h) tma_load_2d(smem_u32(sA + r.s * kABytes + h * 8192), &tmA, k0 + 64 * h, row, fb);
     }
-    if (!ok) {
-      for (int s = 0; s < S; ++s) mbar_wait(smem_u32(&full[s]), 0);
-      if (lane == 0) set_status(c.status, kStatusTimeout);
-    }
   } else if (warp == 1) {
     constexpr uint32_t idesc = mma_idesc(128, BN, true);
     const bool leader = elect_one();
     const uint32_t a0 = desc_mn_lo(smem_u32(sA), 8192), b0 = desc_mn_lo(smem_u32(sB), 8192);
     Ring r;
     for (int st = 0; st < steps; ++st, r.next<S>()) {
-      if (!(ok = mbar_wait(smem_u32(&full[r.s]), r.phase))) break;
+      if (!(ok = st != waits.stop && mbar_wait(smem_u32(&full[r.s]), r.phase, waits.clocks))) break;
       tc_fence_after();
       const uint32_t a = a0 + r.s * (kABytes >> 4), b = b0 + r.s * (Cfg::kBBytes >> 4);
       if (leader) {
@@ -504,11 +514,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
         mma_commit(smem_u32(&empty[r.s]));
       }
     }
+    if (!ok) *reinterpret_cast<volatile int*>(&gave_up) = 1;   // before the epilogue is released
+    __syncwarp();
+    // all products, or those issued before giving up: the epilogue waits for them either way
     if (leader) {
-      if (ok && steps > 0) mma_commit(smem_u32(&done));
+      if (steps > 0) mma_commit(smem_u32(&done));
       else mbar_arrive(smem_u32(&done));
     }
-    if (!ok && lane == 0) set_status(c.status, kStatusTimeout);
   } else if (warp >= 2 && warp < 6) {
     const int t = threadIdx.x - 64;   // 0 .. 127
     if (bias) {
@@ -518,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
       float a = 0.0f, b = 0.0f;
       Ring r;
       for (int st = 0; st < steps; ++st, r.next<S>()) {
-        if (!(ok = mbar_wait(smem_u32(&full[r.s]), r.phase))) break;
+        if (!(ok = mbar_wait(smem_u32(&full[r.s]), r.phase, waits.clocks))) break;
         const unsigned char* tile = sB + r.s * Cfg::kBBytes + (p >> 5) * 8192;
         const int ch = (p & 31) >> 2, in = (p & 3) * 4;   // 16-byte column and byte within it
 #pragma unroll 8
@@ -540,11 +552,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
       }
       if (t < BN && n0 + t < c.N) c.bias_part[(size_t)split * c.N + n0 + t] = sbias[t];
     }
-    const bool got = mbar_wait(smem_u32(&done), 0);
+    const bool got = mbar_wait(smem_u32(&done), 0, kWaitClocks);
     tc_fence_after();
-    if (!got || !ok) {
-      if (lane == 0) set_status(c.status, kStatusTimeout);
-    } else {
+    ok = got && ok;
+    if (ok && !*reinterpret_cast<volatile int*>(&gave_up)) {
       const int q = warp & 3, row = k0 + q * 32 + lane;
       float* out = c.part + ((size_t)split * c.K + row) * c.N + n0;
       for (int n = 0; n < BN; n += 16) {
@@ -577,7 +588,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
       int yb;
       const bf16* p = gather_base(c.g, row0, yb) + off;
       const int y0 = yb + dy;
-      if (!(ok = mbar_wait(smem_u32(&empty[r.s]), r.phase ^ 1))) break;
+      if (!(ok = mbar_wait(smem_u32(&empty[r.s]), r.phase ^ 1, waits.clocks))) break;
       if (tv) {
         uint32_t dst = smem_u32(sA) + r.s * kABytes + (q >> 3) * 8192 + rr * 128;
 #pragma unroll 8
@@ -593,11 +604,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad(const __grid_constant__ C
         r.phase ^= 1;
       }
     }
-    if (!ok && lane == 0) set_status(c.status, kStatusTimeout);
+  }
+  if (!ok && lane == 0) {
+    set_status(c.guard.status, kStatusTimeout);
+    gave_up = 1;
   }
   tc_fence_before();
   __syncthreads();
+  if (gave_up) {   // (otherwise the products have waited for the copies)
+    if (warp == 0) drain_fills<S>(full, filled);
+    __syncthreads();
+  }
   if (warp == 1) {
+    mbar_wait(smem_u32(&done), 0, kWaitClocks);   // (an epilogue that gave up has not waited for the products)
     tc_fence_after();
     tmem_free<kCols>(tmem);
   }
@@ -733,7 +752,7 @@ int configure_conv_kernels() {
 }
 
 int launch_conv_fwd(const void* X, int NV, int Hin, int Cin, const void* W, int Kp, const float* bias, int Cout, void* Y,
-                    int* status, cudaStream_t s) {
+                    Guard guard, cudaStream_t s) {
   CUtensorMap tb;
   if (!tma_map(&tb, W, Cout, Kp, Kp, Cout)) return HR_ERR_CUDA;
   ConvArgs c = {};
@@ -746,12 +765,12 @@ int launch_conv_fwd(const void* X, int NV, int Hin, int Cin, const void* W, int 
   c.C = Cout;
   c.bias = bias;
   c.out = static_cast<bf16*>(Y);
-  c.status = status;
+  c.guard = guard;
   return Cout == 32 ? launch_conv<32, false>(tb, c, s)
                     : (Cout == 64 ? launch_conv<64, false>(tb, c, s) : launch_conv<128, false>(tb, c, s));
 }
 
-int launch_conv_dgrad(const void* dPre, int NV, int Hin, int Cin, const void* wT, int Cout, const void* X, void* dX, int* status,
+int launch_conv_dgrad(const void* dPre, int NV, int Hin, int Cin, const void* wT, int Cout, const void* X, void* dX, Guard guard,
                       cudaStream_t s) {
   CUtensorMap tb;
   const int BN = Cin == 32 ? 32 : 64;   // four taps' accumulators, twice: 8 BN columns
@@ -766,7 +785,7 @@ int launch_conv_dgrad(const void* dPre, int NV, int Hin, int Cin, const void* wT
   c.nkt = Cout / kStep;
   c.out = static_cast<bf16*>(dX);
   c.mask = static_cast<const bf16*>(X);
-  c.status = status;
+  c.guard = guard;
   c.C = Cin;
   c.nblocks = Cin / BN;
   c.nclass = 4;
@@ -789,24 +808,24 @@ int launch_conv_dgrad(const void* dPre, int NV, int Hin, int Cin, const void* wT
 }
 
 int launch_conv_wgrad(const void* X, int NV, int Hin, int Cin, int Kp, const void* dPre, int Cout, float* dW, float* db,
-                      float* part, size_t part_floats, int* status, cudaStream_t s) {
+                      float* part, size_t part_floats, Guard guard, cudaStream_t s) {
   WgradArgs c = {};
   c.g = conv_gather(static_cast<const bf16*>(X), NV, Cin, Hin);
   c.K = Kp;
   c.N = Cout;
-  c.status = status;
+  c.guard = guard;
   const CUtensorMap none = {};
   return launch_wgrad(none, c, static_cast<const bf16*>(dPre), c.g.M, true, dW, db, part, part_floats, s);
 }
 
 int launch_dense_wgrad(const void* x, long long rows, int K, const void* dPre, int N, float* dW, float* db, float* part,
-                       size_t part_floats, int* status, cudaStream_t s) {
+                       size_t part_floats, Guard guard, cudaStream_t s) {
   CUtensorMap ta;
   if (!tma_map(&ta, x, rows, K, K, 64)) return HR_ERR_CUDA;
   WgradArgs c = {};
   c.K = K;
   c.N = N;
-  c.status = status;
+  c.guard = guard;
   return launch_wgrad(ta, c, static_cast<const bf16*>(dPre), rows, false, dW, db, part, part_floats, s);
 }
 

@@ -62,6 +62,20 @@ struct InstRec {
   int st0, nst;        // the instance's sub-tiles
 };
 
+// Bounds of the tensor-core kernels' waits (hr_tcgen05.cuh), and where they report one
+// that ran out
+struct Waits {
+  long long clocks;   // of one wait, in SM clocks
+  int stop;           // the products give up before this K step of a block, as after a wait
+                      // that ran out (-1: never; set by tests of what follows)
+};
+constexpr long long kWaitClocks = 1ll << 31;   // about a second
+constexpr Waits kWaits = {kWaitClocks, -1};
+struct Guard {
+  int* status;
+  Waits waits;
+};
+
 struct Context {
   hr_limits lim;
   // batch layout: n_inst == 1 and vt == nullptr for a single-instance context
@@ -167,6 +181,7 @@ struct Context {
   int ev_ready;
   // status and work counters
   int* status;
+  Waits waits;
   unsigned long long* stats;  // [3][kStatsPer]
 };
 

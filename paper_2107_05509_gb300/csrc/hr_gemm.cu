@@ -17,7 +17,7 @@
 //
 // Every mbarrier wait is bounded (about one second of device time); a wait that
 // runs out sets a status bit, the CTA stops issuing work, waits (bounded) for its own
-// copies in flight, frees its tensor memory and returns.
+// copies and products in flight (drain_fills), frees its tensor memory and returns.
 #include <algorithm>
 #include <mutex>
 
@@ -39,7 +39,7 @@ struct GemmArgs {
   long long split_stride;   // elements between split outputs (split-K partials)
   int out_bf16;
   int rows16;               // every row of a bf16 C starts on 16 bytes
-  int* status;
+  Guard guard;
 };
 
 // 16 columns of a warp's 32 rows (lane: row row0 + lane): bias, ReLU, conversion (bias null
@@ -135,8 +135,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
     int issued = 0;
     for (int kt = 0; kt < nkt; ++kt) {
       const int s = kt % kStages;
-      if (kt >= kStages && !mbar_wait(smem_u32(&empty_bar[s]), ((kt / kStages) + 1) & 1)) {
-        if (lane == 0) set_status(g.status, kStatusTimeout);
+      if (kt >= kStages && !mbar_wait(smem_u32(&empty_bar[s]), ((kt / kStages) + 1) & 1, g.guard.waits.clocks)) {
+        if (lane == 0) set_status(g.guard.status, kStatusTimeout);
         atomicExch(&abort_flag, 1);
         break;
       }
@@ -149,21 +149,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
       }
       ++issued;
     }
-    // copies still in flight must land before the CTA may exit
-    for (int kt = max(0, issued - kStages); kt < issued; ++kt)
-      mbar_wait(smem_u32(&full_bar[kt % kStages]), (kt / kStages) & 1);
+    drain_fills<kStages>(full_bar, issued);   // copies still in flight must land before the CTA may exit
   } else if (warp == 1) {
     // MMA issuer
     constexpr uint32_t idesc = mma_idesc(kBM, BN);
     const bool leader = elect_one();
     const uint32_t a0 = desc_lo(smem_u32(sA)), b0 = desc_lo(smem_u32(sB));
-    bool ok = true;
     for (int kt = 0; kt < nkt; ++kt) {
       const int s = kt % kStages;
-      if (!mbar_wait(smem_u32(&full_bar[s]), (kt / kStages) & 1)) {
-        if (lane == 0) set_status(g.status, kStatusTimeout);
+      if (kt == g.guard.waits.stop || !mbar_wait(smem_u32(&full_bar[s]), (kt / kStages) & 1, g.guard.waits.clocks)) {
+        if (lane == 0) set_status(g.guard.status, kStatusTimeout);
         atomicExch(&abort_flag, 1);
-        ok = false;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -172,16 +168,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
         mma_commit(smem_u32(&empty_bar[s]));   // the stage is free once these MMAs have read it
       }
     }
+    // all products, or those issued before giving up: the epilogue waits for them either way
     if (leader) {
-      if (ok && nkt > 0) mma_commit(smem_u32(&done_bar));
-      else mbar_arrive(smem_u32(&done_bar));   // nothing (more) will be computed: release the epilogue
+      if (nkt > 0) mma_commit(smem_u32(&done_bar));
+      else mbar_arrive(smem_u32(&done_bar));
     }
   } else if (warp >= 2) {
     // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 = tile rows
-    const bool ok = mbar_wait(smem_u32(&done_bar), 0);
+    const bool ok = mbar_wait(smem_u32(&done_bar), 0, kWaitClocks);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (!ok) {
-      set_status(g.status, kStatusTimeout);
+      set_status(g.guard.status, kStatusTimeout);
     } else if (!*reinterpret_cast<volatile int*>(&abort_flag)) {
       const int q = warp & 3;
       const bool split = gridDim.z > 1;
@@ -200,6 +197,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 1) {
+    mbar_wait(smem_u32(&done_bar), 0, kWaitClocks);   // (an epilogue that gave up has not waited for the products)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
@@ -236,9 +234,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   extern __shared__ __align__(1024) unsigned char gsm_raw[];
   unsigned char* sA = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(gsm_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* sB = sA + S * kPairHalf;
-  __shared__ __align__(8) uint64_t full[S], empty[S], acc_full[2], acc_empty[2];
+  __shared__ __align__(8) uint64_t full[S], empty[S], acc_full[2], acc_empty[2], drained;
   __shared__ uint32_t tmem_slot;
+  __shared__ int gave_up, filled[2];   // of the pair (both CTAs write them); filled: the first CTA's
   __shared__ float xpose[8][kXpose];
+  const Waits& waits = g.guard.waits;
   const int warp = warp_id(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const int tm = (g.M + kPairM - 1) / kPairM, tn = (g.N + kPairN - 1) / kPairN, tiles = tm * tn;
@@ -252,6 +252,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       mbar_init(smem_u32(&acc_full[b]), 1);
       mbar_init(smem_u32(&acc_empty[b]), 16);   // the epilogue warps of both CTAs
     }
+    mbar_init(smem_u32(&drained), 1);
+    gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) tmem_alloc_pair<512>(smem_u32(&tmem_slot));
@@ -263,14 +265,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   bool ok = true;
   if (warp == 0) {
     const bool leader = elect_one();
-    int s = 0;
+    int s = 0, issued = 0;
     uint32_t phase = 0;
     for (int t = pair; ok && t < tiles; t += pairs) {
       int m, n;
       pair_tile(t, tm, tn, m, n);
       const int ma = m * kPairM + 128 * (int)rank, nb = n * kPairN + 128 * (int)rank;
       for (int kt = 0; kt < nkt; ++kt) {
-        if (!(ok = mbar_wait(smem_u32(&empty[s]), phase ^ 1))) break;
+        if (!(ok = mbar_wait(smem_u32(&empty[s]), phase ^ 1, waits.clocks))) break;
+        ++issued;
         if (leader) {
           if (rank == 0) mbar_expect_tx(smem_u32(&full[s]), 4 * kPairHalf);
           const uint32_t fb = cluster_addr(smem_u32(&full[s]), 0);
@@ -280,24 +283,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         if (++s == S) s = 0, phase ^= 1;
       }
     }
-    // the products wait for every copy; when a role gave up, a bounded wait for those in flight
-    if (!ok) {
-      if (rank == 0)
-        for (int i = 0; i < S; ++i) mbar_wait(smem_u32(&full[i]), 0);
-      if (lane == 0) set_status(g.status, kStatusTimeout);
-    }
+    if (lane == 0) store_cluster(cluster_addr(smem_u32(&filled[rank]), 0), issued);
   } else if (warp == 1 && rank == 0) {
     constexpr uint32_t idesc = mma_idesc(kPairM, kPairN);
     const bool leader = elect_one();
     const uint32_t a0 = desc_lo(smem_u32(sA)), b0 = desc_lo(smem_u32(sB));
-    int s = 0, it = 0;
+    int s = 0, it = 0, step = 0;
     uint32_t phase = 0;
     for (int t = pair; ok && t < tiles; t += pairs, ++it) {
       const int b = it & 1;
-      if (!(ok = mbar_wait_cluster(smem_u32(&acc_empty[b]), ((it >> 1) & 1) ^ 1))) break;
+      if (!(ok = mbar_wait_cluster(smem_u32(&acc_empty[b]), ((it >> 1) & 1) ^ 1, waits.clocks))) break;
       tc_fence_after();
       for (int kt = 0; kt < nkt; ++kt) {
-        if (!(ok = mbar_wait(smem_u32(&full[s]), phase))) break;
+        if (!(ok = step++ != waits.stop && mbar_wait(smem_u32(&full[s]), phase, waits.clocks))) break;
         tc_fence_after();
         if (leader) {
           mma_step_pair(tmem + b * kPairN, a0 + s * (kPairHalf >> 4), b0 + s * (kPairHalf >> 4), idesc, kt > 0);
@@ -307,7 +305,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       }
       if (ok && leader) mma_commit_pair(smem_u32(&acc_full[b]));
     }
-    if (!ok && lane == 0) set_status(g.status, kStatusTimeout);
   } else if (warp >= 2) {
     const int q = warp & 3, half = warp < 6 ? 0 : kPairN / 2;
     int it = 0;
@@ -316,7 +313,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       int m, n;
       pair_tile(t, tm, tn, m, n);
       const int row0 = m * kPairM + 128 * (int)rank + q * 32;
-      if (!(ok = mbar_wait(smem_u32(&acc_full[b]), (it >> 1) & 1))) break;
+      if (!(ok = mbar_wait(smem_u32(&acc_full[b]), (it >> 1) & 1, waits.clocks))) break;
       tc_fence_after();
       for (int c = half; c < half + kPairN / 2; c += 16) {
         float v[16];
@@ -327,11 +324,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(cluster_addr(smem_u32(&acc_empty[b]), 0));
     }
-    if (!ok && lane == 0) set_status(g.status, kStatusTimeout);
+  }
+  if (!ok && lane == 0) {
+    set_status(g.guard.status, kStatusTimeout);
+    for (uint32_t r = 0; r < 2; ++r) store_cluster(cluster_addr(smem_u32(&gave_up), r), 1);
   }
   tc_fence_before();
   __syncthreads();
   cluster_sync();   // no CTA ends while the other's copies, products or arrivals may reach it
+  if (gave_up) {    // (otherwise the products have waited for the copies, the epilogues for the products)
+    if (warp == 0 && rank == 0) drain_fills<S>(full, max(filled[0], filled[1]));   // both CTAs' copies count here
+    if (warp == 1) {
+      if (rank == 0 && elect_one()) mma_commit_pair(smem_u32(&drained));
+      mbar_wait_cluster(smem_u32(&drained), 0, kWaitClocks);
+    }
+    __syncthreads();
+    cluster_sync();
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_free_pair<512>(tmem);
@@ -430,7 +439,7 @@ int configure_gemm_kernels() {
 }
 
 int launch_gemm(const void* A, int lda, const void* Bm, int ldb, int M, int N, int K, const float* bias, int relu,
-                void* C, int ldc, int out_bf16, int splits, float* split_buf, int* status, cudaStream_t s) {
+                void* C, int ldc, int out_bf16, int splits, float* split_buf, Guard guard, cudaStream_t s) {
   if (M < 1 || N < 1 || K < kBK || K % kBK != 0 || lda < K || ldb < K || lda % 8 || ldb % 8 || splits < 1)
     return HR_ERR_ARG;
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(Bm)) & 15) return HR_ERR_ARG;
@@ -445,7 +454,7 @@ int launch_gemm(const void* A, int lda, const void* Bm, int ldb, int M, int N, i
   g.K = K;
   g.kt_per_split = (kt_total + splits - 1) / splits;
   splits = (kt_total + g.kt_per_split - 1) / g.kt_per_split;
-  g.status = status;
+  g.guard = guard;
   if (splits > 1) {
     if (!split_buf) return HR_ERR_ARG;
     g.bias = nullptr;

@@ -61,7 +61,7 @@ int launch_vertex_error(const float* verts, const float* ref, int V, int n, floa
 // bf16 tensor-core GEMM C = act(A B^T + bias) (hr_gemm.cu); splits > 1 needs
 // split_buf of splits * M * N floats
 int launch_gemm(const void* A, int lda, const void* B, int ldb, int M, int N, int K, const float* bias, int relu,
-                void* C, int ldc, int out_bf16, int splits, float* split_buf, int* status, cudaStream_t s);
+                void* C, int ldc, int out_bf16, int splits, float* split_buf, Guard guard, cudaStream_t s);
 int configure_gemm_kernels();
 
 // the proposal network's 3x3 stride-2 convolutions and weight gradients (hr_conv.cu); all
@@ -70,14 +70,14 @@ int configure_gemm_kernels();
 // dgrad: dX with the ReLU mask of X (needs Cin >= 32, Cout >= 64).  part: scratch.
 int configure_conv_kernels();
 int launch_conv_fwd(const void* X, int NV, int Hin, int Cin, const void* W, int Kp, const float* bias, int Cout, void* Y,
-                    int* status, cudaStream_t s);
+                    Guard guard, cudaStream_t s);
 int launch_conv_dgrad(const void* dPre, int NV, int Hin, int Cin, const void* wT, int Cout, const void* X, void* dX,
-                      int* status, cudaStream_t s);
+                      Guard guard, cudaStream_t s);
 int launch_conv_wgrad(const void* X, int NV, int Hin, int Cin, int Kp, const void* dPre, int Cout, float* dW, float* db,
-                      float* part, size_t part_floats, int* status, cudaStream_t s);
+                      float* part, size_t part_floats, Guard guard, cudaStream_t s);
 // dW [N][K] = dPre^T x, db = column sums of dPre; x [rows][K], dPre [rows][N]
 int launch_dense_wgrad(const void* x, long long rows, int K, const void* dPre, int N, float* dW, float* db, float* part,
-                       size_t part_floats, int* status, cudaStream_t s);
+                       size_t part_floats, Guard guard, cudaStream_t s);
 
 // per-device properties of the render kernels (persistent grid)
 int render_grid(int device, int* blocks, int* threads, int* num_sms);

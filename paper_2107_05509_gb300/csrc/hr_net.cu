@@ -196,6 +196,8 @@ struct Net {
   float* split;          // partial sums of split reductions
   size_t split_floats;
   int* status;
+  Waits waits;
+  Guard guard() const { return Guard{status, waits}; }
 };
 
 Layer make_layer(int N, int K, size_t& off) {
@@ -233,7 +235,7 @@ bool nalloc(T** p, size_t count) {
 
 int gemm(Net* n, const bf16* A, int lda, const bf16* Bm, int ldb, int M, int N, int K, const float* bias, int relu,
          void* C, int ldc, bool out_bf16, cudaStream_t s, int splits = 1) {
-  return launch_gemm(A, lda, Bm, ldb, M, N, K, bias, relu, C, ldc, out_bf16 ? 1 : 0, splits, n->split, n->status, s);
+  return launch_gemm(A, lda, Bm, ldb, M, N, K, bias, relu, C, ldc, out_bf16 ? 1 : 0, splits, n->split, n->guard(), s);
 }
 
 // refresh the bf16 weights and their transposes from the float32 master copy
@@ -256,7 +258,7 @@ int net_forward(Net* n, const float* cams, cudaStream_t s) {
   for (int l = 0; l < kConv; ++l) {
     const Layer& L = n->conv[l];
     if ((rc = launch_conv_fwd(n->act[l], n->NV, kHin[l], kCin[l], n->w16 + L.w, L.K, n->w32 + L.b, L.N, n->act[l + 1],
-                              n->status, s)) != HR_OK)
+                              n->guard(), s)) != HR_OK)
       return rc;
   }
   k_features<<<nblk((long long)n->NV * kZ), 256, 0, s>>>(n->act[kConv], cams, n->NV, n->Z);
@@ -276,7 +278,7 @@ int net_forward(Net* n, const float* cams, cudaStream_t s) {
 // gradients of a dense layer y = act(W x + b) given dPre = dL/d(W x + b) [rows][N]:
 // db = column sums, dW [N][K] = dPre^T x (x [rows][K]); dx = dPre W
 int dense_bwd(Net* n, const Layer& L, int li, const bf16* dPre, const bf16* x, int rows, bf16* dx, cudaStream_t s) {
-  const int rc = launch_dense_wgrad(x, rows, L.K, dPre, L.N, n->g32 + L.w, n->g32 + L.b, n->split, n->split_floats, n->status, s);
+  const int rc = launch_dense_wgrad(x, rows, L.K, dPre, L.N, n->g32 + L.w, n->g32 + L.b, n->split, n->split_floats, n->guard(), s);
   if (rc != HR_OK) return rc;
   return gemm(n, dPre, L.N, n->wT[li], L.N, rows, L.K, L.N, nullptr, 0, dx, L.K, true, s);
 }
@@ -302,10 +304,10 @@ int net_backward(Net* n, const float* d_out, cudaStream_t s) {
   for (int l = kConv - 1; l >= 0; --l) {
     const Layer& L = n->conv[l];
     if ((rc = launch_conv_wgrad(n->act[l], n->NV, kHin[l], kCin[l], L.K, dPre, L.N, n->g32 + L.w, n->g32 + L.b, n->split,
-                                n->split_floats, n->status, s)) != HR_OK)
+                                n->split_floats, n->guard(), s)) != HR_OK)
       return rc;
     if (l == 0) break;
-    if ((rc = launch_conv_dgrad(dPre, n->NV, kHin[l], kCin[l], n->wT[l], L.N, n->act[l], next, n->status, s)) != HR_OK) return rc;
+    if ((rc = launch_conv_dgrad(dPre, n->NV, kHin[l], kCin[l], n->wT[l], L.N, n->act[l], next, n->guard(), s)) != HR_OK) return rc;
     std::swap(dPre, next);
   }
   return HR_OK;
@@ -338,6 +340,7 @@ int hr_net_create(int B, int views, hr_net** out) {
   n->B = B;
   n->nv = views;
   n->NV = B * views;
+  n->waits = kWaits;
   size_t off = 0;
   for (int l = 0; l < kConv; ++l) n->conv[l] = make_layer(kCout[l], kKp[l], off);
   n->fv = make_layer(kHid, kZ, off);
@@ -451,6 +454,12 @@ int hr_net_adam(hr_net* net, float lr, float beta1, float beta2, float eps, int 
   int rc = hr::launch_adam(n->w32, n->g32, n->m, n->v, (int)n->P, lr, beta1, beta2, eps, step, s);
   if (rc != HR_OK) return rc;
   return hr::refresh_weights(n, s);
+}
+
+// bounds of the waits of this network's products (tests)
+int hr_internal_net_waits(hr_net* net, int64_t clocks, int stop) {
+  reinterpret_cast<hr::Net*>(net)->waits = hr::Waits{clocks, stop};
+  return HR_OK;
 }
 
 int hr_net_status(hr_net* net, hr_stream stream) {

@@ -37,22 +37,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// bounded wait for the phase of `parity` to complete (2^31 clocks, about a second); false
-// when it ran out.  The bound is on the SM's clock: reading the global timer between two
-// tries held up the wake-up.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+// bounded wait for the phase of `parity` to complete; false when it ran out.  The bound is
+// on the SM's clock: reading the global timer between two tries held up the wake-up.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long clocks) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   for (;;) {
 #pragma unroll 1
     for (int i = 0; i < 16; ++i)
       if (mbar_try_wait(bar, parity)) return true;
-    if (clock64() - t0 > (1ll << 31)) return false;
+    if (clock64() - t0 > clocks) return false;
   }
 }
 
 // the same for arrivals from the other CTA of a cluster
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, long long clocks) {
   const long long t0 = clock64();
   for (;;) {
     uint32_t ok;
@@ -62,8 +61,25 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
         : "r"(bar), "r"(parity)
         : "memory");
     if (ok) return true;
-    if (clock64() - t0 > (1ll << 31)) return false;
+    if (clock64() - t0 > clocks) return false;
   }
+}
+
+// When a wait has run out, its role stops, the others' waits run out likewise, and no
+// block may end, nor its tensor memory be freed, before the copies and the products that
+// are under way are done:
+//   the copies: fill n of a ring of S slots is in slot n % S and completes phase n / S of
+//   its barrier.  Of `issued` fills the last S can be under way; each is waited for in its
+//   own phase (a slot is filled again only when the fill before it has been used, so no
+//   older phase is open), all of them for `kWaitClocks` at most: a fill that another
+//   role shares in and never made completes no phase, and its copy has landed by then.
+//   the products: a last commit, by the thread that issued them, on a barrier of its own.
+template <int S>
+__device__ __forceinline__ void drain_fills(uint64_t* full, int issued) {
+  const long long t0 = clock64();
+  for (int n = issued > S ? issued - S : 0; n < issued; ++n)
+    while (!mbar_try_wait(smem_u32(&full[n % S]), (n / S) & 1))
+      if (clock64() - t0 > kWaitClocks) return;
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
@@ -139,6 +155,9 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 }
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void store_cluster(uint32_t cluster_addr, int v) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
