@@ -150,6 +150,35 @@ def test_edge_samples_do_not_depend_on_their_lanes(B_, name, samples):
     assert B_.hr_get_status(ctx) == B_.HR_OK
 
 
+@pytest.mark.parametrize("width", [100, 16])
+def test_edge_samples_of_a_hand_alone_and_among_others(B_, width):
+    """One hand's samples, alone (four lanes each) and in batches whose numbers of samples
+    take the rule to two lanes and to one: the hand's fixed-point gradient has the same
+    bits, with the silhouettes' lists (100 columns) and with sub-tiles of more candidates
+    than a list holds, whose rays go through the tree (16)."""
+    sc, h = scene("ragged"), hand()
+    f, samples = width / sc.W, 777
+    H = int(sc.H * f)
+    cams = np.array(sc.cams, np.float32, copy=True)
+    cams[:, :4] *= f    # fx, fy, cx, cy
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a, np.float32), device="cuda")
+    rng = np.random.default_rng(width)
+    bg, adj = rng.random((sc.N * H * width, 3)), rng.normal(size=(sc.N * H * width, 3))
+    model, outs = B_.Model(h), []
+    for n in (1, 24, 48):   # 2331, 55944 and 111888 samples
+        bt = B_.Batch(h.V, h.F, h.E, [(sc.N, width, H, 2, samples, i) for i in range(n)])
+        many = lambda a: t(np.concatenate([a] * n))
+        verts, img, out = many(sc.verts[None]), torch.empty((bt.total_pixels, 3), device="cuda"), torch.empty((n, h.V, 3), device="cuda")
+        o = B_.render_opts(seed=7, flags=B_.HR_DETERMINISTIC | B_.HR_BWD_REUSE_FWD | B_.HR_BWD_NO_INTERIOR)
+        cam_t, bg_t, adj_t = many(cams), many(bg), many(adj)
+        B_.hr_build_bvh_batch(bt, model, verts)
+        B_.hr_render_fwd_batch(bt, model, verts, cam_t, bg_t, o, img)
+        B_.hr_render_bwd_batch(bt, model, verts, cam_t, bg_t, o, adj_t, out)
+        assert B_.hr_get_status(bt) == B_.HR_OK
+        outs.append(out[0].clone())
+    assert outs[0].abs().max() > 0 and all(torch.equal(outs[0], o) for o in outs[1:])
+
+
 @pytest.mark.parametrize("width", [208, 104, 56, 24])
 def test_lists_of_every_length(B_, width):
     """Sub-tiles of a hand seen ever smaller: lists of up to 32, 64, 128 and more records
