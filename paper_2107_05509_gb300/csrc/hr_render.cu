@@ -124,6 +124,50 @@ __device__ __forceinline__ void isect(const float4* __restrict__ tris, int k, fl
   }
 }
 
+// One node of a closest-hit traversal; false when there is no next one.
+template <bool STATS>
+__device__ __forceinline__ bool visit_node(const Node* __restrict__ nodes, const float4* __restrict__ tris, float3 o,
+                                           float3 d, float3 inv, Hit& h, int (&stack)[kStack], int& sp, int& node,
+                                           int* status, Counts& cnt) {
+  const float4* np = reinterpret_cast<const float4*>(nodes + node);
+  if (STATS) ++cnt.nodes;
+  float4 a = __ldg(np), b = __ldg(np + 1), c = __ldg(np + 2);
+  int4 dd = __ldg(reinterpret_cast<const int4*>(np + 3));
+  float tl, tr;
+  bool hl = slab(a.x, a.y, a.z, a.w, b.x, b.y, o, inv, h.t, tl);
+  bool hrr = slab(b.z, b.w, c.x, c.y, c.z, c.w, o, inv, h.t, tr);
+  if (hl && dd.x < 0) {
+    isect<STATS>(tris, ~dd.x, o, d, h, cnt);
+    hl = false;
+  }
+  if (hrr && dd.y < 0) {
+    isect<STATS>(tris, ~dd.y, o, d, h, cnt);
+    hrr = false;
+  }
+  if (hl && hrr) {
+    int nearc = dd.x, farc = dd.y;
+    if (tr < tl) {
+      nearc = dd.y;
+      farc = dd.x;
+    }
+    if (sp < kStack) {
+      stack[sp++] = farc;
+    } else {
+      set_status(status, kStatusLimit);
+    }
+    node = nearc;
+  } else if (hl) {
+    node = dd.x;
+  } else if (hrr) {
+    node = dd.y;
+  } else {
+    if (sp == 0) return false;
+    node = stack[--sp];
+  }
+  return true;
+}
+__device__ __forceinline__ float3 slab_inv(float3 d) { return make_float3(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z)); }
+
 // Closest hit against the LBVH (root = internal node 0); ties in t go to the lower
 // triangle id.  At most `max_visits` internal nodes are visited (a well-formed tree
 // never needs more than F - 1); past it the status records a limit error.
@@ -131,7 +175,7 @@ template <bool STATS>
 __device__ Hit trace(const Node* __restrict__ nodes, const float4* __restrict__ tris, float3 o, float3 d,
                      int* status, Counts& cnt, int max_visits) {
   Hit h{-1, INFINITY, 0.0f, 0.0f};
-  float3 inv = make_float3(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
+  const float3 inv = slab_inv(d);
   int stack[kStack];
   int sp = 0;
   int node = 0;
@@ -140,41 +184,7 @@ __device__ Hit trace(const Node* __restrict__ nodes, const float4* __restrict__ 
       set_status(status, kStatusLimit);
       break;
     }
-    const float4* np = reinterpret_cast<const float4*>(nodes + node);
-    if (STATS) ++cnt.nodes;
-    float4 a = __ldg(np), b = __ldg(np + 1), c = __ldg(np + 2);
-    int4 dd = __ldg(reinterpret_cast<const int4*>(np + 3));
-    float tl, tr;
-    bool hl = slab(a.x, a.y, a.z, a.w, b.x, b.y, o, inv, h.t, tl);
-    bool hrr = slab(b.z, b.w, c.x, c.y, c.z, c.w, o, inv, h.t, tr);
-    if (hl && dd.x < 0) {
-      isect<STATS>(tris, ~dd.x, o, d, h, cnt);
-      hl = false;
-    }
-    if (hrr && dd.y < 0) {
-      isect<STATS>(tris, ~dd.y, o, d, h, cnt);
-      hrr = false;
-    }
-    if (hl && hrr) {
-      int nearc = dd.x, farc = dd.y;
-      if (tr < tl) {
-        nearc = dd.y;
-        farc = dd.x;
-      }
-      if (sp < kStack) {
-        stack[sp++] = farc;
-      } else {
-        set_status(status, kStatusLimit);
-      }
-      node = nearc;
-    } else if (hl) {
-      node = dd.x;
-    } else if (hrr) {
-      node = dd.y;
-    } else {
-      if (sp == 0) break;
-      node = stack[--sp];
-    }
+    if (!visit_node<STATS>(nodes, tris, o, d, inv, h, stack, sp, node, status, cnt)) break;
   }
   return h;
 }
@@ -1164,10 +1174,29 @@ constexpr int kGradWin = 16;
 struct GradTile {
   WarpTile w;
   float4 hit[kGradWin][32];   // (triangle, u, v, -); with a texture then (cell, fx, fy, k)
+  __device__ __forceinline__ WarpTile& tile() { return w; }
+  __device__ __forceinline__ float4& at(int j) { return hit[j][threadIdx.x & 31]; }
+};
+// the same with each lane's hits in its own (local) memory: the shaders' 41 KB of shared
+// memory per block would leave the tree's traversal (k_overflow) a quarter of the SM's L1
+struct OverflowTile {
+  WarpTile& w;
+  float4 hit[kGradWin];
+  __device__ __forceinline__ explicit OverflowTile(WarpTile& t) : w(t) {}
+  __device__ __forceinline__ WarpTile& tile() { return w; }
+  __device__ __forceinline__ float4& at(int j) { return hit[j]; }
 };
 
+// direction of sample s of this lane's pixel
+__device__ __forceinline__ float3 sample_dir(const RenderArgs& a, const WarpTile& wt, int s) {
+  const int lane = threadIdx.x & 31, px = wt.t.x0 + (lane % kSubW), py = wt.t.y0 + (lane / kSubW);
+  float u1, u2;
+  jitter(a, wt.t.ctr1, wt.t.W, px, py, s, u1, u2);
+  return primary_dir(wt.cam, __fadd_rn((float)px, u1), __fadd_rn((float)py, u2));
+}
+
 // Differentiation of one window (any lanes), samples s0 ..: `pend` = those of this lane
-// with a hit in gt.hit, G = upstream gradient x light colour.
+// with a hit in gt.at(), G = upstream gradient x light colour.
 //
 // At a fixed ray, moving corner k by dp moves the hit's (u, v, t) by -M^-1 (w_k dp) with
 // M = [e1, e2, -d] and weights w = (1 - u - v, u, v), so
@@ -1184,14 +1213,13 @@ struct GradTile {
 // triangle whose |cos| to the view is below kGrazing takes the first form, with each
 // sample's own direction (made again) and so its own rounding.
 constexpr float kGrazing = 1.0f / 32;
-template <bool STATS, class Sum>
-__device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, unsigned pend, int s0, float3 G, Sum sum,
+template <bool STATS, class Sum, class Tile>
+__device__ __forceinline__ void grad_window(const RenderArgs& a, Tile& gt, unsigned pend, int s0, float3 G, Sum sum,
                                             Counts& cnt) {
-  const int lane = threadIdx.x & 31;
   const unsigned all = pend;
-  const float3 o = make_float3(gt.w.cam.c[0], gt.w.cam.c[1], gt.w.cam.c[2]);
+  const float3 o = make_float3(gt.tile().cam.c[0], gt.tile().cam.c[1], gt.tile().cam.c[2]);
   while (pend) {
-    const int tri = __float_as_int(gt.hit[__ffs(pend) - 1][lane].x);
+    const int tri = __float_as_int(gt.at(__ffs(pend) - 1).x);
     const float4* rec = a.frec + (size_t)kFaceRec * tri;
     const float4 r0 = __ldg(rec), r1 = __ldg(rec + 1), r2 = __ldg(rec + 2), r3 = __ldg(rec + 3), r4 = __ldg(rec + 4),
                  r5 = __ldg(rec + 5), r6 = __ldg(rec + 6), r8 = __ldg(rec + 8);
@@ -1199,7 +1227,7 @@ __device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, u
     unsigned m = 0u;
     for (unsigned q = pend; q; q &= q - 1u) {
       const int j = __ffs(q) - 1;
-      if (__float_as_int(gt.hit[j][lane].x) == tri) m |= 1u << j;
+      if (__float_as_int(gt.at(j).x) == tri) m |= 1u << j;
     }
     pend &= ~m;
     const float3 n0 = xyz(r0), n1 = xyz(r1), n2 = xyz(r2);
@@ -1217,7 +1245,7 @@ __device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, u
     while (m) {
       const int j = __ffs(m) - 1;
       m &= m - 1u;
-      const float4 hj = gt.hit[j][lane];
+      const float4 hj = gt.at(j);
       if (STATS) ++cnt.hits;
       const float u = hj.y, v = hj.z, w[3] = {__fsub_rn(__fsub_rn(1.0f, u), v), u, v};
       const float3 nm = interp_normal(u, v, n0, n1, n2);
@@ -1238,7 +1266,7 @@ __device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, u
         gu = __fmaf_rn(dux, __fsub_rn(t01.z, t01.x), __fmul_rn(duy, __fsub_rn(t01.w, t01.y)));
         gv = __fmaf_rn(dux, __fsub_rn(r8.x, t01.x), __fmul_rn(duy, __fsub_rn(r8.y, t01.y)));
         galb = lerp_rn(lerp_rn(t00, t10, ts.fx), lerp_rn(t0y, t1y, ts.fx), ts.fy);
-        if (a.d_tex) gt.hit[j][lane] = make_float4(__int_as_float(ts.cell), ts.fx, ts.fy, k);
+        if (a.d_tex) gt.at(j) = make_float4(__int_as_float(ts.cell), ts.fx, ts.fy, k);
       } else {
         gu = __fmul_rn(k, cu);
         gv = __fmul_rn(k, cv);
@@ -1256,11 +1284,8 @@ __device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, u
       }
       float gn = __fmaf_rn(gu, u, __fmul_rn(gv, v));
       if (grazing) {
-        const WarpTile& wt = gt.w;
-        const int px = wt.t.x0 + (lane % kSubW), py = wt.t.y0 + (lane / kSubW);
-        float u1, u2;
-        jitter(a, wt.t.ctr1, wt.t.W, px, py, s0 + j, u1, u2);
-        const float3 d = primary_dir(wt.cam, __fadd_rn((float)px, u1), __fadd_rn((float)py, u2));
+        const WarpTile& wt = gt.tile();
+        const float3 d = sample_dir(a, wt, s0 + j);
         const float3 dxe2 = dcross(d, e2), e1xd = dcross(e1, d), q = comb(gu, dxe2, gv, e1xd);
         const float invD = 1.0f / vdot(e1, dxe2);
         gu = __fmul_rn(q.x, invD);
@@ -1293,11 +1318,11 @@ __device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, u
   if (!a.d_tex) return;
   // texel gradients, cell by cell: the four corners' sums of weight x k, times G
   for (pend = all; pend;) {
-    const int cell = __float_as_int(gt.hit[__ffs(pend) - 1][lane].x);
+    const int cell = __float_as_int(gt.at(__ffs(pend) - 1).x);
     float wt[4] = {0.f, 0.f, 0.f, 0.f};
     for (unsigned q = pend; q; q &= q - 1u) {
       const int j = __ffs(q) - 1;
-      const float4 hj = gt.hit[j][lane];
+      const float4 hj = gt.at(j);
       if (__float_as_int(hj.x) != cell) continue;
       pend &= ~(1u << j);
       const float ky = hj.w * hj.z, k0 = hj.w - ky;
@@ -1318,58 +1343,95 @@ __device__ __forceinline__ void grad_window(const RenderArgs& a, GradTile& gt, u
 
 // hits of samples [s0, s0 + S) of this lane's pixel into window entries j0 .. (all lanes
 // call it; `live` lanes take part); returns the lane's entries with a hit
-template <bool STATS, int S, bool TRACE>
-__device__ __forceinline__ unsigned trace_samples(const RenderArgs& a, GradTile& gt, int off, int K, unsigned m0,
+template <bool STATS, int S, class Tile>
+__device__ __forceinline__ unsigned trace_samples(const RenderArgs& a, Tile& gt, int off, int K, unsigned m0,
                                                   int s0, int j0, bool live, Counts& cnt) {
-  const int lane = threadIdx.x & 31;
-  const WarpTile& wt = gt.w;
-  const int px = wt.t.x0 + (lane % kSubW), py = wt.t.y0 + (lane / kSubW);
   float3 d[S];
   Hit h[S];
 #pragma unroll
   for (int j = 0; j < S; ++j) {
-    float u1, u2;
-    jitter(a, wt.t.ctr1, wt.t.W, px, py, s0 + j, u1, u2);
-    d[j] = primary_dir(wt.cam, __fadd_rn((float)px, u1), __fadd_rn((float)py, u2));
+    d[j] = sample_dir(a, gt.tile(), s0 + j);
     if (STATS && live) {
       ++cnt.samples;
       ++cnt.rays;
     }
   }
-  if (K > 0) {
-    closest_staged<STATS, S>(a, gt.w, off, K, m0, live, d, h, cnt);
-  } else {
-    const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      h[j] = Hit{-1, INFINITY, 0.0f, 0.0f};
-      if (TRACE && live) h[j] = trace<STATS>(a.nodes, a.tris, o, d[j], a.status, cnt, a.max_visits);
-    }
-  }
+  closest_staged<STATS, S>(a, gt.tile(), off, K, m0, live, d, h, cnt);
   unsigned hits = 0u;
 #pragma unroll
   for (int j = 0; j < S; ++j) {
     if (h[j].tri < 0) continue;
-    gt.hit[j0 + j][lane] = make_float4(__int_as_float(h[j].tri), h[j].u, h[j].v, 0.0f);
+    gt.at(j0 + j) = make_float4(__int_as_float(h[j].tri), h[j].u, h[j].v, 0.0f);
     hits |= 1u << (j0 + j);
   }
   return hits;
 }
 
+// the same without a candidate list, samples [s0, s0 + n) into window entries 0 ..: a lane
+// goes on with its next ray when it is done with one, so that the warp waits for the
+// lanes' sums of nodes and not for the longest of 32 traversals n times.  With the hits in
+// the lanes' own memory: backward of 5 views of 125 x 336, 52 spp, 6 k triangles 596 -> 509
+// us in all, of 14 views of 152 x 256, 57 spp, 24.6 k triangles 1777 -> 1560.
+template <bool STATS, class Tile>
+__device__ __forceinline__ unsigned traverse_samples(const RenderArgs& a, Tile& gt, int s0, int n, bool live, Counts& cnt) {
+  const WarpTile& wt = gt.tile();
+  for (int j = 0; j < n; ++j) {   // the directions, in the hits' places
+    const float3 d = sample_dir(a, wt, s0 + j);
+    gt.at(j) = make_float4(d.x, d.y, d.z, 0.0f);
+    if (STATS && live) {
+      ++cnt.samples;
+      ++cnt.rays;
+    }
+  }
+  const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
+  unsigned hits = 0u;
+  Hit h{-1, INFINITY, 0.0f, 0.0f};
+  float3 d = o, inv = o;
+  int stack[kStack];
+  int sp = 0, node = 0, visits = 0, j = live ? -1 : n;
+  bool next = true;
+  while (j < n) {
+    if (next) {
+      if (j >= 0 && h.tri >= 0) {
+        gt.at(j) = make_float4(__int_as_float(h.tri), h.u, h.v, 0.0f);
+        hits |= 1u << j;
+      }
+      if (++j == n) break;
+      d = xyz(gt.at(j));
+      inv = slab_inv(d);
+      h = Hit{-1, INFINITY, 0.0f, 0.0f};
+      sp = node = visits = 0;
+    }
+    if (visits++ >= a.max_visits) {   // as in trace()
+      set_status(a.status, kStatusLimit);
+      next = true;
+    } else {
+      next = !visit_node<STATS>(a.nodes, a.tris, o, d, inv, h, stack, sp, node, a.status, cnt);
+    }
+  }
+  __syncwarp();
+  return hits;
+}
+
 // Gradient of samples [s0, s1) of this lane's pixel (upstream g, `live` lanes only; all
-// lanes call it after stage_tile), traced S at a time.  The windows and the order of a
-// window's sums depend on [s0, s1) alone.
-template <bool STATS, int S, class Sum, bool TRACE = true>
-__device__ __forceinline__ void grad_samples(const RenderArgs& a, GradTile& gt, int off, int K, unsigned m0,
+// lanes call it after stage_tile), traced S at a time, or (TRACE) ray by ray where there
+// is no candidate list.  The windows and the order of a window's sums depend on [s0, s1)
+// alone.
+template <bool STATS, int S, class Sum, bool TRACE, class Tile>
+__device__ __forceinline__ void grad_samples(const RenderArgs& a, Tile& gt, int off, int K, unsigned m0,
                                              int s0, int s1, bool live, float3 g, Sum sum, Counts& cnt) {
   const float3 G = make_float3(g.x * a.sh.lrgb.x, g.y * a.sh.lrgb.y, g.z * a.sh.lrgb.z);
   for (int w0 = s0; w0 < s1; w0 += kGradWin) {
     const int n = min(kGradWin, s1 - w0);
     unsigned pend = 0u;
-    int j = 0;
-    for (; j + S <= n; j += S) pend |= trace_samples<STATS, S, TRACE>(a, gt, off, K, m0, w0 + j, j, live, cnt);
-    if (S > 1)
-      for (; j < n; ++j) pend |= trace_samples<STATS, 1, TRACE>(a, gt, off, K, m0, w0 + j, j, live, cnt);
+    if (TRACE && K <= 0) {
+      pend = traverse_samples<STATS>(a, gt, w0, n, live, cnt);
+    } else {
+      int j = 0;
+      for (; j + S <= n; j += S) pend |= trace_samples<STATS, S>(a, gt, off, K, m0, w0 + j, j, live, cnt);
+      if (S > 1)
+        for (; j < n; ++j) pend |= trace_samples<STATS, 1>(a, gt, off, K, m0, w0 + j, j, live, cnt);
+    }
     grad_window<STATS>(a, gt, pend, w0, G, sum, cnt);
     __syncwarp();
   }
@@ -2254,20 +2316,16 @@ __global__ void __launch_bounds__(kRenderThreads, kFwdMinBlocks) k_shade_fwd(Ren
   flush_counts<STATS>(cnt, stats);
 }
 
-struct FwdTile {
-  WarpTile w;
-};
 template <bool STATS>
-__device__ __forceinline__ void overflow_grad(const RenderArgs& a, GradTile& gt, int inst, int off, int K, unsigned m0, int s0, int s1, bool live, float3 g, Counts& cnt) {
-  if (a.wk.det)
-    grad_samples<STATS, 1>(a, gt, off, K, m0, s0, s1, live, g,
-                           SumWide<unsigned long long>{a.wk.fx + (size_t)inst * 6 * a.V}, cnt);
-  else
-    grad_samples<STATS, 1>(a, gt, off, K, m0, s0, s1, live, g, SumF32{a.wk.extra + (size_t)inst * 8 * a.V}, cnt);
+__device__ __forceinline__ void overflow_grad(const RenderArgs& a, OverflowTile& gt, int inst, int off, int K, unsigned m0,
+                                              int s0, int s1, bool live, float3 g, Counts& cnt) {
+  if (a.wk.det) {
+    typedef SumWide<unsigned long long> Sum;
+    grad_samples<STATS, 1, Sum, true>(a, gt, off, K, m0, s0, s1, live, g, Sum{a.wk.fx + (size_t)inst * 6 * a.V}, cnt);
+  } else {
+    grad_samples<STATS, 1, SumF32, true>(a, gt, off, K, m0, s0, s1, live, g, SumF32{a.wk.extra + (size_t)inst * 8 * a.V}, cnt);
+  }
 }
-template <bool STATS>   // the forward overflow kernel never takes this branch
-__device__ __forceinline__ void overflow_grad(const RenderArgs&, FwdTile&, int, int, int, unsigned, int, int, bool,
-                                              float3, Counts&) {}
 
 // The rare paths, kept out of the gather and the shaders so that their registers are
 // sized for their own work: (1) sub-tiles whose work items did not fit their
@@ -2280,10 +2338,9 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
                                                                                      const float* __restrict__ adjoint,
                                                             float* __restrict__ image, unsigned long long* stats) {
   pdl_wait();
-  typedef typename std::conditional<BWD, GradTile, FwdTile>::type Tile;
-  __shared__ Tile tiles[kWarps];
-  Tile& gt = tiles[threadIdx.x >> 5];
-  WarpTile& wt = gt.w;
+  __shared__ WarpTile tiles[kWarps];
+  WarpTile& wt = tiles[threadIdx.x >> 5];
+  OverflowTile gt(wt);   // (backward)
   const RenderArgs a0 = with_iter(a_in);
   const int total = subtile_count(a0);
   const int n = (int)min(*reinterpret_cast<volatile unsigned*>(&a0.wk.ctr[2 + 2 * a0.n_inst]), (unsigned)total);
@@ -2296,8 +2353,7 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
     const RenderArgs a = for_inst(a0, t.inst);
     int2 pk = a.wk.st[st];
     if (pk.y > 0 && !in_range(a.status, (long long)pk.x + pk.y - 1, 0, a.wk.pool_cap)) pk.y = -1;
-    const Cam cam = load_cam(a.cams, t.view);
-    if (BWD) {
+    if constexpr (BWD) {
       // in the items' chunks too: each chunk's sums are added exactly as its work item
       // would add them, so fixed-point sums do not depend on which sub-tiles overflowed
       bool live;
@@ -2346,10 +2402,9 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
     item = a0.wk.items[slot];
     if (!load_item(a0, item, t, pk) || pk.y >= 0) continue;
     const RenderArgs a = for_inst(a0, t.inst);
-    const Cam cam = load_cam(a.cams, t.view);
     int s0, s1;
     item_samples(item.y, item.z, t.spp, s0, s1);
-    if (BWD) {
+    if constexpr (BWD) {
       bool live;
       const float3 g = lane_adjoint(a, t, adjoint, live);
       unsigned m0;
