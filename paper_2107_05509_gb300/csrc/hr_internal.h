@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "hr_device.cuh"
 
 namespace hr {
@@ -78,6 +80,13 @@ int launch_conv_wgrad(const void* X, int NV, int Hin, int Cin, int Kp, const voi
 // dW [N][K] = dPre^T x, db = column sums of dPre; x [rows][K], dPre [rows][N]
 int launch_dense_wgrad(const void* x, long long rows, int K, const void* dPre, int N, float* dW, float* db, float* part,
                        size_t part_floats, Guard guard, cudaStream_t s);
+
+// SMs of the current device
+inline int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 152;
+  return std::max(n, 1);
+}
 
 // per-device properties of the render kernels (persistent grid)
 int render_grid(int device, int* blocks, int* threads, int* num_sms);

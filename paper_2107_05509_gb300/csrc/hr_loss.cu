@@ -671,7 +671,7 @@ int launch_resample(const typename Acc::Value* src, int N, int H, int W, int Ho,
   const int threads = std::min(kResampleThreads, (C * Wo + 31) / 32 * 32), segments = (C * Wo + threads - 1) / threads;
   // more rows per block once there are eight blocks per SM without
   const int per_block = (int)std::min<long long>(
-      Ho, std::max<long long>({1, std::min<long long>(rows * segments / (8 * 152), kResampleRows), rows * segments / 0x7fffffff + 1}));
+      Ho, std::max<long long>({1, std::min<long long>(rows * segments / (8 * sm_count()), kResampleRows), rows * segments / 0x7fffffff + 1}));
   const unsigned groups = (unsigned)((Ho + per_block - 1) / per_block), grid = (unsigned)((long long)N * groups * segments);
   // columns' ranges of at most two pixels (up to twice the size, or exactly half) need two
   if (W <= Wo || W == 2 * Wo)

@@ -3205,12 +3205,12 @@ int launch_render_bwd(Context* ctx, const hr_model* m, const float* verts, const
     if (rc != HR_OK) return rc;
     tm.end(kTimeBwdSil);
     // At most edge_lanes lanes per edge sample, fewer when the samples alone fill the GPU
-    // (about 2.5 times its resident threads at this kernel's registers): the lanes of a
+    // (about 2.5 times an SM's resident threads at this kernel's registers): the lanes of a
     // sample share its search but each do its set-up.  Whole passes at 4 / 2 / 1 lanes, us:
     // 28 k samples 326 / 326 / 347, 40 k 323 / 329 / 335, 78 k 278 / 267 / 267, 86 k with
     // long lists 1795 / 1692 / 1714; this kernel for a batch of 64 hands 2177 / 1712 / 1404.
     int L = ctx->tune.edge_lanes;
-    while (L > 1 && (long long)nv * Ne * L > 200000) L >>= 1;
+    while (L > 1 && (long long)nv * Ne * L > 1316LL * ctx->num_sms) L >>= 1;
     const long long n = ((long long)nv * Ne + 32 / L - 1) / (32 / L) * 32;
     const unsigned grid = (unsigned)((n + kRenderThreads - 1) / kRenderThreads);
     tm.begin(kTimeBwdEdges);

@@ -225,13 +225,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// SMs of the current device
-inline int sm_count() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 152;
-  return std::max(n, 1);
-}
-
 // 2-D bf16 tensor map over rows x cols (cols contiguous, row pitch ld elements) with
 // boxes of 64 columns x box_rows, 128-byte swizzle; values outside are zero (hr_gemm.cu)
 bool tma_map(CUtensorMap* map, const void* ptr, long long rows, int cols, int ld, int box_rows);
