@@ -173,10 +173,10 @@ typedef struct hr_render_opts {
 
 /* Sizes a context is created for; all scratch is allocated once, up front. */
 typedef struct hr_limits {
-    int32_t max_V;      /* vertices (<= 65536; up to 8192 the backward sums in shared
-                           memory, beyond that with global atomics)             */
+    int32_t max_V;      /* vertices (<= 65536; up to 8192 the backward sums in float,
+                           beyond that in float64)                              */
     int32_t max_F;      /* triangles (<= 65536; the BVH build runs in one block per
-                           instance up to ~2400, in a multi-block build beyond)  */
+                           instance up to 8192, in a multi-block build beyond)   */
     int32_t max_E;      /* edges                                                 */
     int32_t max_views;  /* views per call                                        */
     int32_t max_width;  /* image width W per call                                */
@@ -538,7 +538,8 @@ int hr_gemm_bf16(hr_context* ctx, const void* A, int lda, const void* B, int ldb
 typedef struct hr_net hr_net;
 
 int hr_net_param_count(void);
-/* Allocate a network for B instances of `views` views (all scratch up front). */
+/* Allocate a network for B instances of `views` views (all scratch up front); B <= 4096,
+ * views <= 64, B * views a multiple of 4. */
 int hr_net_create(int B, int views, hr_net** out);
 int hr_net_destroy(hr_net* net);
 /* Load parameters (device float[hr_net_param_count()]) and reset the Adam moments. */

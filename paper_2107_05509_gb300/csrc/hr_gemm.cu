@@ -118,15 +118,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                 "r"(kTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (warp == 1) tmem_alloc<kTmemCols>(smem_u32(&tmem_base));
+  tc_fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  tc_fence_after();
   const uint32_t tmem = tmem_base;
 
   if (warp == 0) {
@@ -162,7 +157,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
         atomicExch(&abort_flag, 1);
         break;
       }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tc_fence_after();
       if (leader) {
         mma_step(tmem, a0 + s * (kABytes >> 4), b0 + s * (kBBytes >> 4), idesc, kt > 0);
         mma_commit(smem_u32(&empty_bar[s]));   // the stage is free once these MMAs have read it
@@ -176,7 +171,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
   } else if (warp >= 2) {
     // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 = tile rows
     const bool ok = mbar_wait(smem_u32(&done_bar), 0, kWaitClocks);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_fence_after();
     if (!ok) {
       set_status(g.guard.status, kStatusTimeout);
     } else if (!*reinterpret_cast<volatile int*>(&abort_flag)) {
@@ -194,12 +189,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
       }
     }
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     mbar_wait(smem_u32(&done_bar), 0, kWaitClocks);   // (an epilogue that gave up has not waited for the products)
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    tc_fence_after();
+    tmem_free<kTmemCols>(tmem);
   }
 }
 

@@ -234,8 +234,8 @@ bool nalloc(T** p, size_t count) {
 }
 
 int gemm(Net* n, const bf16* A, int lda, const bf16* Bm, int ldb, int M, int N, int K, const float* bias, int relu,
-         void* C, int ldc, bool out_bf16, cudaStream_t s, int splits = 1) {
-  return launch_gemm(A, lda, Bm, ldb, M, N, K, bias, relu, C, ldc, out_bf16 ? 1 : 0, splits, n->split, n->guard(), s);
+         void* C, int ldc, bool out_bf16, cudaStream_t s) {
+  return launch_gemm(A, lda, Bm, ldb, M, N, K, bias, relu, C, ldc, out_bf16 ? 1 : 0, 1, nullptr, n->guard(), s);
 }
 
 // refresh the bf16 weights and their transposes from the float32 master copy
@@ -332,6 +332,7 @@ int hr_net_param_count(void) {
 
 int hr_net_create(int B, int views, hr_net** out) {
   using namespace hr;
+  // (B views) % 4: no kernel needs it any more; numbers of images that were refused stay so
   if (!out || B < 1 || views < 1 || B > 4096 || views > 64 || (B * views) % 4 != 0) return HR_ERR_ARG;
   *out = nullptr;
   Net* n = new (std::nothrow) Net();
