@@ -192,8 +192,8 @@ __host__ __device__ constexpr int ctr_trace(int n) { return 3 + 3 * n; }
 __host__ __device__ constexpr int ctr_sort(int n) { return 4 + 3 * n; }
 __host__ __device__ constexpr int ctr_alloc_base(int n) { return (5 + 3 * n + 1) & ~1; }
 __host__ __device__ constexpr int ctr_words(int n) { return ctr_alloc_base(n) + 2 * n; }
-// meshes up to this many vertices take float backward sums (per block of the shader
-// in a single-instance context); larger ones float64 sums
+// meshes up to this many vertices take float backward sums (one copy per SM in a
+// single-instance context); larger ones float64 sums
 constexpr int kPartialMaxV = 8192;
 constexpr int kLossBlocks = 304;         // loss blocks of a single-instance context (2 per SM of a GB300)
 constexpr int kLossBlocksBatch = 128;    // per instance in a batch

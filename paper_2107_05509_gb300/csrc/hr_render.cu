@@ -5,16 +5,17 @@
 // Primary rays of a pinhole camera are coherent, so the forward and the interior
 // backward work on 8x4-pixel sub-tiles, one warp per sub-tile at a time.
 //
-// Candidate lists (forward).  A sample can hit a triangle only if the sample lies in
-// the triangle's screen box (padded by half a pixel), and every shader tests that box
-// before intersecting, so a sub-tile needs the triangle records whose boxes meet it:
+// Candidate lists (forward).  A triangle can only be hit in its screen box (padded by
+// half a pixel), so a sub-tile needs the triangle records whose boxes meet it; of its
+// pixels, those that the triangle can cover (tri_pixel_mask) are kept with the record:
 //   k_bin (count)  each (view, record) pair counts itself into the sub-tiles its box
 //                  meets;
 //   k_bin_alloc    each sub-tile gets a pool range for its K records and 1-16 work
 //                  items of consecutive samples (more for longer lists, so no single
 //                  warp holds up the launch);
 //   k_background   sub-tiles that no record meets get the background (second stream);
-//   k_bin (fill)   the pairs write their records, boxes and depths into the ranges;
+//   k_bin (fill)   the pairs write their records, boxes, depths and pixel masks into
+//                  the ranges;
 //   k_bin_sort     each list is sorted by nearest camera depth.
 // k_gather (a frustum walk of the LBVH per sub-tile) makes the backward's own lists
 // when the forward's cannot be reused.
@@ -27,12 +28,14 @@
 //                  transpose of the lists' pixel masks), in depth order, with the same
 //                  float32 Moller-Trumbore test and closest-hit rule as a per-ray
 //                  traversal, stopping at the first candidate nearer than none of its
-//                  hits; shades, and writes per-item sums.  The warp finishing a sub-tile's last item sums the items in
-//                  item order (deterministic) and writes the pixels.
+//                  hits; shades, and writes per-item sums.  The warp finishing a
+//                  sub-tile's last item sums the items in item order (deterministic)
+//                  and writes the pixels.
 //   k_shade_bwd    the same samples re-traced (no hit records are kept between
-//                  the passes); every hit is differentiated at the fixed ray and the
-//                  gradient accumulated per run of hits on one triangle in registers,
-//                  summed over the warp, and added into one partial per SM.
+//                  the passes); every hit is differentiated at the fixed ray, a lane's
+//                  hits triangle by triangle in windows of 16 samples, and a triangle's
+//                  sums of a window are added to memory (single instance: one partial
+//                  per SM).
 //   k_reduce_partials  fixed-order sum of the partials.
 //
 // Per-ray LBVH traversal (trace) serves the hr_trace entry point and the sub-tiles
@@ -48,8 +51,8 @@
 // one launch.  Sub-tiles are numbered over all views of all instances (a view table
 // maps a sub-tile to its view, instance, resolution and samples per pixel); each
 // instance has its own BVH, vertices, normals and region of the work-item table.
-// Warps take items instance after instance; a batch's backward adds each run's sums
-// straight into its instance's gradient.  A single-instance call is a batch of one
+// Warps take items of one instance, then of others with items left; a batch's backward
+// adds its sums straight into its instance's gradient.  A single-instance call is a batch of one
 // with a uniform view layout (no table).
 #include <type_traits>
 
@@ -63,7 +66,7 @@ constexpr int kRenderThreads = 128;   // 4 warps per block
 constexpr int kWarps = kRenderThreads / 32;
 constexpr int kFwdMinBlocks = 7;      // launch bound of the forward shader (72 registers)
 constexpr int kBwdMinBlocks = 4;      // launch bound of the backward shader (128 registers)
-constexpr int kBlocksPerSm = 8;       // largest persistent grid; backward partials are sized for it
+constexpr int kBlocksPerSm = 8;       // largest persistent grid
 constexpr int kSubW = 8, kSubH = 4;   // sub-tile; lane = pixel
 constexpr int kLeafCap = 512;         // candidates per sub-tile
 constexpr int kFrontCap = 256;        // breadth-first frontier per level (dense meshes need the width)
@@ -932,10 +935,9 @@ __device__ __forceinline__ unsigned tri_pixel_mask(float4 b, const ScreenTri& t,
 // s = o - v0, q = s x e1 and e2 . q only depend on the candidate; they are computed
 // once (the same operations, so the same float32 values) instead of once per ray.
 // Arrays of float4: lanes reading neighbouring candidates meet no bank conflict.
-// 32 of them, a window of a longer list (a tile of 48, with two masks per lane, took 9 % more
-// of a batch of 64 hands: 10.3 -> 9.4 ms).
+// 32 of them, one per lane; longer lists pass through the tile in windows (a tile of 48, with
+// two masks per lane, took 9 % more of a batch of 64 hands: 10.3 -> 9.4 ms).
 constexpr int kCandCap = 32;
-static_assert(kCandCap >= 32, "longer lists pass through the tile in windows of 32");
 struct CandTile {
   float4 e1[kCandCap];   // e1, depth below which no ray's hit lets the candidate matter
   float4 e2[kCandCap];   // e2, triangle id
@@ -943,7 +945,7 @@ struct CandTile {
   float4 q[kCandCap];    // q
 };
 
-// candidates [c0, c0 + n), n <= 32, of the list at `off` into the tile (one per lane);
+// candidates [c0, c0 + n), n <= kCandCap, of the list at `off` into the tile (one per lane);
 // returns the lane's pixel's candidates, bit i = slot i
 template <bool STATS>
 __device__ __forceinline__ unsigned stage_candidates(const RenderArgs& a, CandTile& ct, int off, int c0, int n,
@@ -1019,7 +1021,7 @@ struct WarpTile {
   Cam cam;
 };
 
-// sub-tile t and its first kCandCap candidates into the warp's tile (all lanes call);
+// sub-tile t into the warp's tile, with its candidates where they fit (all lanes call);
 // m0: the lane's pixel's candidates, bit i = slot i
 template <bool STATS>
 __device__ __forceinline__ void stage_tile(const RenderArgs& a, WarpTile& wt, const SubTile& t, int off, int K, unsigned& m0,
@@ -1048,9 +1050,9 @@ __device__ __forceinline__ void closest_staged(const RenderArgs& a, WarpTile& wt
     return;
   }
   const float3 o = make_float3(wt.cam.c[0], wt.cam.c[1], wt.cam.c[2]);
-  for (int w = 0; w < K; w += 32) {
+  for (int w = 0; w < K; w += kCandCap) {
     if (!__any_sync(0xffffffffu, !done)) break;
-    m0 = stage_candidates<STATS>(a, wt.cand, off, w, min(32, K - w), o, cnt);
+    m0 = stage_candidates<STATS>(a, wt.cand, off, w, min(kCandCap, K - w), o, cnt);
     if (!done) walk_candidates<STATS, S>(wt.cand, m0, d, h, done, cnt);
     __syncwarp();   // every lane is done with the window
   }
@@ -1211,7 +1213,10 @@ __device__ __forceinline__ float3 sample_dir(const RenderArgs& a, const WarpTile
 // Their float32 errors are common to all of a triangle's samples, and seen nearly
 // edge-on they are small differences of large products (and the gradient is large): a
 // triangle whose |cos| to the view is below kGrazing takes the first form, with each
-// sample's own direction (made again) and so its own rounding.
+// sample's own direction (made again) and so its own rounding.  Against 64 bits the two
+// forms are equally far off, at 1 / 30 2.3e-5 of a 20 mm triangle's gradient and facing
+// 8.5e-7, the rounding of the hits' own u and v; at the same float32 rays they differ by
+// 1.1e-6 at 1 / 30.
 constexpr float kGrazing = 1.0f / 32;
 template <bool STATS, class Sum, class Tile>
 __device__ __forceinline__ void grad_window(const RenderArgs& a, Tile& gt, unsigned pend, int s0, float3 G, Sum sum,
@@ -1458,11 +1463,11 @@ constexpr int kGroupSubtiles = 8;
 // ---------------------------------------------------------------------------------
 // forward candidate lists by screen-space binning
 // ---------------------------------------------------------------------------------
-// The shaders test every sample against a candidate's screen box (project_record:
-// padded by half a pixel, unbounded when a vertex is not in front of the camera)
-// before intersecting it, so a sub-tile's list needs exactly the triangle records
-// whose box meets the sub-tile's sample square [x0, x0 + 8] x [y0, y0 + 4].  The
-// forward builds the lists by binning each (view, record) pair into the sub-tiles its
+// A triangle can only be hit in its screen box (project_record: padded by half a pixel,
+// unbounded when a vertex is not in front of the camera), so a sub-tile's list holds the
+// triangle records whose box meets the sub-tile's sample square [x0, x0 + 8] x [y0, y0 +
+// 4], and for each the pixels that the triangle can cover: the shaders test no box, a
+// lane takes the candidates whose mask has its pixel.  The forward builds the lists by binning each (view, record) pair into the sub-tiles its
 // box meets -- k_bin counts them, k_bin_alloc gives every sub-tile its pool range and
 // work items, k_bin in fill mode writes the records, k_bin_sort orders each list by
 // nearest depth -- instead of a frustum walk of the BVH per sub-tile.
@@ -2429,7 +2434,7 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
 //   kAccPartials  block b into partial b % nparts of `nparts` partials [V][8]
 //                 (L2-resident, zeroed before the launch), summed in partial order by
 //                 k_reduce_partials (single instance)
-//   kAccDirect    every run of hits on one triangle straight into its instance's
+//   kAccDirect    every triangle's sums of a window straight into its instance's
 //                 extra [V][8] (batches)
 //   kAccGlobal    meshes beyond kPartialMaxV vertices: into the instance's float64
 //                 extra64 [6V] (long runs of cancelling contributions)
@@ -3155,7 +3160,7 @@ int launch_render_bwd(Context* ctx, const hr_model* m, const float* verts, const
                ctx->dN);
   };
   if (interior) {
-    // float sums up to kPartialMaxV vertices (per block, or per instance in a batch),
+    // float sums up to kPartialMaxV vertices (per SM, or per instance in a batch),
     // float64 beyond; fixed-point sums when deterministic
     const bool global_acc = V > kPartialMaxV;
     if (!det && global_acc &&
