@@ -481,9 +481,10 @@ __device__ __forceinline__ void add3(T* dst, int i, float x, float y, float z) {
 // round(x 2^40) (two's complement in an unsigned word); integer addition is exact and
 // associative, so the sums do not depend on the order of the atomics.
 constexpr double kFixScale = 1099511627776.0;   // 2^40
-__device__ __forceinline__ void add_fixed(unsigned long long* p, float x) {
-  atomicAdd(p, (unsigned long long)__double2ll_rn((double)x * kFixScale));
+__device__ __forceinline__ unsigned long long to_fixed(float x) {
+  return (unsigned long long)__double2ll_rn((double)x * kFixScale);
 }
+__device__ __forceinline__ void add_fixed(unsigned long long* p, float x) { atomicAdd(p, to_fixed(x)); }
 template <>
 __device__ __forceinline__ void add3<unsigned long long>(unsigned long long* dst, int i, float x, float y, float z) {
   add_fixed(&dst[3 * i], x);
@@ -1128,7 +1129,8 @@ __device__ __forceinline__ void write_pixel(const RenderArgs& a, const SubTile& 
 // sums as [V][3] then [V][3].
 struct SumF32 {
   float* p;
-  __device__ __forceinline__ void add(int V, int i, float3 dv, float3 dn) const {
+  __device__ __forceinline__ unsigned sharing(int) const { return 0u; }
+  __device__ __forceinline__ void add(int V, int i, float3 dv, float3 dn, unsigned) const {
     float* q = p + 8 * (size_t)i;
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(q), "f"(dv.x), "f"(dv.y), "f"(dv.z), "f"(0.0f)
                  : "memory");
@@ -1136,15 +1138,46 @@ struct SumF32 {
                  : "memory");
   }
 };
-template <class T>
-struct SumWide {   // double, or unsigned long long (fixed point)
-  T* p;
-  __device__ __forceinline__ void add(int V, int i, float3 dv, float3 dn) const {
+struct SumF64 {
+  double* p;
+  __device__ __forceinline__ unsigned sharing(int) const { return 0u; }
+  __device__ __forceinline__ void add(int V, int i, float3 dv, float3 dn, unsigned) const {
     add3(p, i, dv.x, dv.y, dv.z);
     add3(p + 3 * V, i, dn.x, dn.y, dn.z);
   }
 };
-
+// Fixed point: one copy of the sums for all SMs, so lanes that differentiate one triangle
+// side by side, twelve or more of them, are summed first (whole numbers: the sums' bits are
+// the same).  Without, large triangles at few samples waited for their vertices' atomics: one
+// view of 2048^2 (4096^2) at 1 spp 165 -> 102 (724 -> 188) us; below twelve the lanes' sums
+// cost more than the atomics (8 x 512x384 at 16 spp: 188, with groups from six lanes 198).
+constexpr int kShared = 12;
+struct SumFixed {
+  unsigned long long* p;
+  // the lanes here that are on this triangle, when there are enough of them
+  __device__ __forceinline__ unsigned sharing(int tri) const {
+    const unsigned lanes = __match_any_sync(__activemask(), tri);
+    return __popc(lanes) >= kShared ? lanes : 0u;
+  }
+  __device__ __forceinline__ void add(int V, int i, float3 dv, float3 dn, unsigned lanes) const {
+    if (!lanes) {
+      add3(p, i, dv.x, dv.y, dv.z);
+      add3(p + 3 * V, i, dn.x, dn.y, dn.z);
+      return;
+    }
+    const float x[6] = {dv.x, dv.y, dv.z, dn.x, dn.y, dn.z};
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      // in pieces of 26, 26 and 12 bits, whose sums over 32 lanes fit a word
+      const unsigned long long f = to_fixed(x[c]);
+      const unsigned lo = __reduce_add_sync(lanes, (unsigned)f & 0x3ffffffu);
+      const unsigned mid = __reduce_add_sync(lanes, (unsigned)(f >> 26) & 0x3ffffffu);
+      const unsigned hi = __reduce_add_sync(lanes, (unsigned)(f >> 52));
+      if ((threadIdx.x & 31) == __ffs(lanes) - 1)
+        atomicAdd(p + (c < 3 ? 3 * i + c : 3 * V + 3 * i + c - 3), lo + ((unsigned long long)mid << 26) + ((unsigned long long)hi << 52));
+    }
+  }
+};
 
 // Value arithmetic of the backward, every contraction spelled out: a window's sums are
 // the same in every kernel that differentiates it (HR_DETERMINISTIC relies on it).
@@ -1313,11 +1346,12 @@ __device__ __forceinline__ void grad_window(const RenderArgs& a, Tile& gt, unsig
       inv = -1.0f;
     }
     const int iv[3] = {__float_as_int(r0.w), __float_as_int(r1.w), __float_as_int(r2.w)};
+    const unsigned sharing = sum.sharing(tri);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       float3 dv = comb(__fmul_rn(su[k], inv), A, __fmul_rn(sv[k], inv), B);
       addmul(dv, __fmul_rn(sn[k], inv), N);
-      sum.add(a.V, iv[k], dv, dn[k]);
+      sum.add(a.V, iv[k], dv, dn[k], sharing);
     }
   }
   if (!a.d_tex) return;
@@ -2325,8 +2359,7 @@ template <bool STATS>
 __device__ __forceinline__ void overflow_grad(const RenderArgs& a, OverflowTile& gt, int inst, int off, int K, unsigned m0,
                                               int s0, int s1, bool live, float3 g, Counts& cnt) {
   if (a.wk.det) {
-    typedef SumWide<unsigned long long> Sum;
-    grad_samples<STATS, 1, Sum, true>(a, gt, off, K, m0, s0, s1, live, g, Sum{a.wk.fx + (size_t)inst * 6 * a.V}, cnt);
+    grad_samples<STATS, 1, SumFixed, true>(a, gt, off, K, m0, s0, s1, live, g, SumFixed{a.wk.fx + (size_t)inst * 6 * a.V}, cnt);
   } else {
     grad_samples<STATS, 1, SumF32, true>(a, gt, off, K, m0, s0, s1, live, g, SumF32{a.wk.extra + (size_t)inst * 8 * a.V}, cnt);
   }
@@ -2479,11 +2512,11 @@ __global__ void __launch_bounds__(kRenderThreads, kBwdMinBlocks) k_shade_bwd(Ren
     int s0, s1;
     item_samples(item.y, item.z, gt.w.t.spp, s0, s1);
     if constexpr (ACC == kAccGlobal)
-      grad_samples<STATS, S, SumWide<double>, false>(a, gt, off, K, m0, s0, s1, live, g,
-                                                     SumWide<double>{a0.wk.extra64 + (size_t)inst * 6 * a0.V}, cnt);
+      grad_samples<STATS, S, SumF64, false>(a, gt, off, K, m0, s0, s1, live, g,
+                                                     SumF64{a0.wk.extra64 + (size_t)inst * 6 * a0.V}, cnt);
     else if constexpr (ACC == kAccFixed)
-      grad_samples<STATS, S, SumWide<unsigned long long>, false>(
-          a, gt, off, K, m0, s0, s1, live, g, SumWide<unsigned long long>{a0.wk.fx + (size_t)inst * 6 * a0.V}, cnt);
+      grad_samples<STATS, S, SumFixed, false>(
+          a, gt, off, K, m0, s0, s1, live, g, SumFixed{a0.wk.fx + (size_t)inst * 6 * a0.V}, cnt);
     else
       grad_samples<STATS, S, SumF32, false>(
           a, gt, off, K, m0, s0, s1, live, g,

@@ -49,3 +49,38 @@ def test_gradients_of_several_windows(levels, W, H, spp):
             fixed.append(dv.clone())
     assert torch.equal(*fixed)
     assert B.hr_get_status(ctx) == B.HR_OK
+
+
+@pytest.mark.parametrize("zoom,spp", [(2.0, 1), (30.0, 1), (30.0, 2), (30.0, 17), (300.0, 1)])
+@pytest.mark.parametrize("size", [1e-6, 1.0, 1e4])
+def test_fixed_point_sums_of_lanes_that_share_a_triangle(zoom, spp, size):
+    """From many triangles per sub-tile to one under the whole image: fixed-point sums
+    (a contribution is rounded to 2^-40) against the oracle at gradients of either sign
+    and a range of sizes, the same bits again when other warps do the same work."""
+    require_gpu()
+    from paper_2107_05509_gb300 import binding as B
+    h, (W, H), seed = _hand(0), (72, 52), 13
+    cfg = I.SceneConfig("shared", views=1, width=W, height=H, spp=spp, edge_samples=0, elevation_deg=20.0, azimuths_deg=(10.0,))
+    verts = oracle.skin(h, I.gt_params(5).astype(np.float32)).astype(np.float32)
+    cams = I.pack_cameras(I.make_cameras(cfg, verts[h.faces[700]].mean(0)))
+    cams[:, 0:2] *= zoom
+    normals = oracle.vertex_normals(verts, h.faces, h.vf_offsets, h.vf_faces)
+    bg = I.background(5, 1, H, W)
+    A = (np.random.default_rng(6).normal(size=(1, H, W, 3)) * size).astype(np.float32)
+    common = dict(spp=spp, edge_samples=0, ka=I.K_AMBIENT, kd=I.K_DIFFUSE, light_dir=I.LIGHT_DIR, light_rgb=I.LIGHT_RGB)
+    ref, _ = oracle.render_bwd(h, verts, cams, H, W, bg, oracle.make_opts(seed=seed, edge_eps=I.EDGE_EPS_PX, **common), A, normals=normals)
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+    model, ctx = B.Model(h), B.Context(h.V, h.F, h.E, 1, W, H)
+    vt, ct, bt, At, img, dv = t(verts), t(cams), t(bg), t(A), torch.empty((1, H, W, 3), device="cuda"), torch.empty((h.V, 3), device="cuda")
+    go = B.render_opts(seed=seed, edge_eps_px=I.EDGE_EPS_PX, flags=B.HR_DETERMINISTIC | B.HR_BWD_REUSE_FWD, **common)
+    B.hr_build_bvh(ctx, model, vt)
+    B.hr_render_fwd(ctx, model, vt, ct, H, W, bt, go, img)
+    fixed = []
+    for blocks in (4, 1):
+        ctx.set_tuning(bwd_blocks_per_sm=blocks)
+        B.hr_render_bwd(ctx, model, vt, ct, H, W, bt, go, At, dv)
+        fixed.append(dv.clone())
+    assert np.abs(ref).max() > 0 and torch.equal(*fixed)
+    if np.abs(ref).max() < 2.0 ** 22:   # (sums wrap at 2^23: 64 bits of 2^-40)
+        assert grad_ok(dv.cpu().numpy(), ref).all()
+    assert B.hr_get_status(ctx) == B.HR_OK
