@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(const __grid_cons
 // and holds 128 rows of the accumulator; one thread of the first CTA issues the products
 // of both (cta_group::2).  A 128 x 128 tile reads 128 bytes of shared memory per clock,
 // all that an SM has, and asks L2 for 20 TB/s; the pair's reads 64 and asks for half.
-// 8192^3 bf16: 775 -> 574 us, 98 % of cuBLAS's burst rate on this chip.  The two
+// 8192^3 bf16: 775 -> 582 us, 97 % of cuBLAS's burst rate on this chip.  The two
 // accumulators (all 512 columns) alternate, so that a tile's epilogue runs
 // beside the next tile's products; CTA pairs take tiles in turn, eight tile rows at a
 // time, which keeps the operands that they share in L2.
@@ -382,7 +382,7 @@ EncodeTiledFn encode_fn() {
 }
 
 // Pairs where there is a tile for nearly every pair and a reduction long enough to cover
-// the coarser last round.  Measured, 128 x 128 tiles -> pairs, us: 8192^3 758 -> 574,
+// the coarser last round.  Measured, 128 x 128 tiles -> pairs, us: 8192^3 758 -> 582,
 // 4096^3 106 -> 84, 3072 x 3072 x 2048 35.2 -> 28.7, 2048 x 2048 x 2048 (64 tiles) 18.5 ->
 // 18.0; but 1792 x 1792 x 2048 (49 tiles) 18.7 -> 19.0, 2304 x 2304 x 512 (81) 16.7 -> 17.6
 // and 3072 x 3072 x 128 14.4 -> 16.4.

@@ -2311,11 +2311,11 @@ __device__ __forceinline__ void finish_item(const RenderArgs& a, const SubTile& 
 
 // warps take work items; S samples per lane at a time.  The sub-tile's description, its
 // camera and its candidates are kept in the warp's shared memory from item to item.
-// Bound by instruction issue (52 % active, 20 of 32 lanes) with the latency of the
-// items' chains beside it.  Against a walk that took every candidate's box and record
-// through shuffles and global loads for each group of samples: 64 M -> 36 M warp
-// instructions and 112 -> 75 us on 8 x 512x384 at 16 spp; 64 hands, 612 views: 6.45 ->
-// 3.30 ms; 1024 views of 256^2 at 4 spp, whose items hold one sample: 2.52 -> 0.98 ms.
+// Bound by instruction issue (50 % active, 20 of 32 lanes, 31 M warp instructions on 8 x
+// 512x384 at 16 spp) with the latency of the items' chains beside it.  Against a walk that
+// took every candidate's box and record through shuffles and global loads for each group
+// of samples: 106 -> 59 us there; 64 hands, 612 views: 6.45 -> 2.99 ms; 1024 views of 256^2
+// at 4 spp, whose items hold one sample: 2.52 -> 0.90 ms.
 template <bool STATS, int S>
 __global__ void __launch_bounds__(kRenderThreads, kFwdMinBlocks) k_shade_fwd(RenderArgs a_in, float* __restrict__ image,
                                                                              unsigned long long* stats) {
@@ -2473,10 +2473,11 @@ __global__ void __launch_bounds__(kRenderThreads, BWD ? kBwdMinBlocks : 8) k_ove
 //                 extra64 [6V] (long runs of cancelling contributions)
 //   kAccFixed     HR_DETERMINISTIC: into the instance's fixed-point sums fx [6V]
 //                 (order-free integer atomics)
-// Bound by instruction issue and the latency of divergent loads.  With the hits of a
-// window differentiated triangle by triangle instead of run by run, the candidates from
-// the tile and vertices summed 16 bytes at a time: 64 hands, 612 views 7.4 -> 4.9 ms
-// (with the edge kernel beside it), textured 16 x 1024^2 at 64 spp 4.5 -> 3.0 ms.
+// Bound by instruction issue (51 % active, 17 of 32 lanes on 8 x 512x384 at 16 spp) and the
+// latency of divergent loads.  With the hits of a window differentiated triangle by
+// triangle instead of run by run, the candidates from the tile and vertices summed 16 bytes
+// at a time: 120 -> 70 us there; 64 hands, 612 views 7.4 -> 3.9 ms (with the edge kernel
+// beside it), textured 16 x 1024^2 at 64 spp 4.5 -> 2.8 ms.
 constexpr int kAccPartials = 0, kAccDirect = 1, kAccGlobal = 2, kAccFixed = 3;
 template <bool STATS, int ACC, int S>
 __global__ void __launch_bounds__(kRenderThreads, kBwdMinBlocks) k_shade_bwd(RenderArgs a_in,
