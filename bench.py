@@ -47,9 +47,9 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # FP32 FMA peak: SMs (read from the device) x 128 FP32 lanes x 2 flop x clock
 LANES = 128
 # modelled FP32 work: per ray made (jitter, screen point, direction), per BVH node
-# visited (two child boxes against a sub-tile frustum or a ray), per candidate
-# screen-box test, per Moller-Trumbore test, per shaded hit (forward) or
-# differentiated hit (backward)
+# visited (two child boxes against a sub-tile frustum or a ray), per candidate read by a
+# sub-tile's warp or tested against an edge ray, per Moller-Trumbore test, per shaded hit
+# (forward) or differentiated hit (backward)
 FLOP_RAY, FLOP_NODE, FLOP_CAND, FLOP_TRI, FLOP_HIT, FLOP_HIT_GRAD = 40, 60, 4, 50, 60, 250
 S_SAMPLES, S_RAYS, S_NODES, S_TRIS, S_HITS, S_CANDS = range(6)
 FLOP_TRACE_NODE, FLOP_EDGE = 40, 120   # per-ray traversal node (two slab tests); edge-sample set-up

@@ -593,7 +593,8 @@ int hr_silhouettes(hr_context* ctx, const hr_model* model, const float* verts, c
  * `stream`, copy 18 counters to host `out` and clear them.  out[0..5] = forward,
  * out[6..11] = the interior backward, out[12..17] = the edge-sample rays, each
  * (estimator samples resolved, rays made individually, BVH nodes visited,
- * Moller-Trumbore tests, hits, candidate screen-box tests).  A sample is resolved
+ * Moller-Trumbore tests, hits, candidates read by a sub-tile's warp or tested against
+ * an edge ray).  A sample is resolved
  * without its own ray when no triangle's screen box meets its sub-tile (the forward)
  * or its sub-tile's frustum misses the scene (the backward's own lists). */
 int hr_get_stats(hr_context* ctx, uint64_t* out, hr_stream stream);

@@ -668,8 +668,8 @@ def hr_silhouettes(ctx, model, verts, cams, lists, counts, stream=None):
 def hr_get_stats(ctx, stream=None):
     """Work counters [3][6] (forward, interior backward, edge rays) x (estimator
     samples resolved, rays made individually, BVH nodes visited, Moller-Trumbore
-    tests, hits, candidate screen-box tests) accumulated by calls made with
-    HR_STATS; cleared on read."""
+    tests, hits, candidates read by a sub-tile's warp or tested against an edge ray)
+    accumulated by calls made with HR_STATS; cleared on read."""
     out = (ctypes.c_uint64 * 18)()
     _check("hr_get_stats", lib().hr_get_stats(ctx.handle, out, _stream(stream)))
     return np.array(out[:], np.uint64).reshape(3, 6)
