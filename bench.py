@@ -58,8 +58,8 @@ KERNEL_NAMES = {"fwd_gather": "k_bin_*", "fwd_shade": "k_shade_fwd", "bwd_gather
 # DRAM bytes (read + write) per launch from the ncu capture summarised under profiles/,
 # with the hash of the render kernels' sources at that capture: a kernel whose source
 # has changed since reports no traffic
-NCU_TRAFFIC = {"k_shade_bwd": (4073472, "a7c40670d9635f27"), "k_shade_fwd": (2200064, "a7c40670d9635f27"),
-               "k_edge_samples": (2942464, "a7c40670d9635f27")}
+NCU_TRAFFIC = {"k_shade_bwd": (4102144, "ab1ad039d8ecf768"), "k_shade_fwd": (2198272, "ab1ad039d8ecf768"),
+               "k_edge_samples": (2940672, "ab1ad039d8ecf768")}
 NCU_TRAFFIC_SOURCES = ("paper_2107_05509_gb300/csrc/hr_render.cu", "paper_2107_05509_gb300/csrc/hr_device.cuh")
 
 
@@ -431,7 +431,7 @@ def run_handrt(args):
             "launch_ms": round(kt_mean[dom], 4), "flops_per_launch": float(kflops[dom]),
             "peak_note": f"FP32 FMA peak: {n_sm} SMs (cudaDevAttrMultiProcessorCount) x {LANES} lanes x 2 flop x "
                          f"{pk.get('sm_max_mhz', 2070.0):.0f} MHz (max SM clock, {pk_kind} clock data)",
-            "flop_model": f"{FLOP_RAY}/ray made + {FLOP_CAND}/candidate box test + {FLOP_TRI}/Moller-Trumbore "
+            "flop_model": f"{FLOP_RAY}/ray made + {FLOP_CAND}/candidate read + {FLOP_TRI}/Moller-Trumbore "
                           f"test + {FLOP_HIT}/shaded hit or {FLOP_HIT_GRAD}/differentiated hit; "
                           f"{FLOP_NODE}/frustum node visit",
             "kernel_ms": {k: round(v, 4) for k, v in kt_mean.items()},

@@ -679,8 +679,9 @@ __global__ void k_vertex_normals(const float* __restrict__ verts_all, const int*
 
 // ---------------------------------------------------------------------------------
 // Multi-block build for meshes whose keys do not fit one block's shared memory (F above
-// 8192): the same Morton codes, hierarchy and refit over global memory, one instance per grid row, the keys sorted by a bitonic
-// network whose stages below 2048 run in shared memory.
+// 8192): the same Morton codes, hierarchy and refit over global memory, one instance per
+// grid row, the keys sorted by a bitonic network whose stages below 2048 run in shared
+// memory.
 // ---------------------------------------------------------------------------------
 constexpr int kSortChunk = 2048;    // keys sorted per block in shared memory
 constexpr int kGridThreads = 256;

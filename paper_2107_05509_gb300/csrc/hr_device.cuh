@@ -201,7 +201,7 @@ constexpr int kLossBlocksBatch = 128;    // per instance in a batch
 __host__ __device__ constexpr int kLossStride(int blocks) { return 4 * blocks + 8; }
 // float4 words of a face's shading record (write_face_record in hr_render.cu)
 constexpr int kFaceRec = 9;
-constexpr int kStatsPer = 6;   // samples, rays, BVH nodes, triangle tests, hits, candidate box tests
+constexpr int kStatsPer = 6;   // samples, rays, BVH nodes, triangle tests, hits, candidates read
 constexpr int kSkinBlocks = 64;
 constexpr int kSkinAcc = 16 * 12 + 10 + 3;   // dA_j (J=16 x 3x4), dbeta, dtau
 constexpr int kMaxJ = 16;

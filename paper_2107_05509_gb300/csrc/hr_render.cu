@@ -103,8 +103,8 @@ __device__ __forceinline__ float safe_inv(float d) {
 }
 
 // work counters of the statistics build (HR_STATS): estimator samples resolved,
-// rays made individually, BVH nodes visited, Moller-Trumbore tests, hits, candidate
-// screen-box tests
+// rays made individually, BVH nodes visited, Moller-Trumbore tests, hits, candidates read
+// by a sub-tile's warp or tested against an edge ray
 struct Counts {
   unsigned samples = 0, rays = 0, nodes = 0, tris = 0, hits = 0, cands = 0;
 };
